@@ -49,33 +49,31 @@ REASON_BITS = {
 # Counters of the sweep kernels measured with ncu (summaries in profiles/), each with
 # the hash of the kernel sources it was measured on; a counter whose hash differs from
 # the current sources is reported as stale (and the fractions built on it as null).
-SWEEP_SOURCES = ["paper_1212_3975_gb300/csrc/ws_bodies.cuh", "paper_1212_3975_gb300/csrc/sweep_ws.cu",
-                 "paper_1212_3975_gb300/csrc/sweep_kernels.cu"]
+SWEEP_SOURCES = ["paper_1212_3975_gb300/csrc/" + f for f in
+                 ("sweep_body.cuh", "sweep_small.cuh", "sweep_launch.cuh", "sweep_kernels.cu")]
 COUNTERS = {
-    # Ising 64x64, p = 1024: 147 blocks of 7 chains, one per SM (the idle lanes of each
-    # warp issue too, so these counts are per attempt of a real chain):
+    # Ising 64x64, p = 1024 (128 blocks of four groups of two chains):
     # profiles/ising_ws_sweep_L64_p1024.md
-    "ising_L64": {"source": "8c638c33e6db10d8", "inst_per_attempt": 8.508,
-                  "shared_wavefronts_per_attempt": 1.013, "traffic_bytes_per_launch": 2565120,
-                  "chains_per_block": 7},
-    # Ising 64x64, compact staging, two blocks per SM (p = 9728):
+    "ising_L64": {"source": "9d3df190ad49e213", "inst_per_attempt": 2.898, "shared_wavefronts_per_attempt": 0.391,
+                  "traffic_bytes_per_launch": 647936},
+    # Ising 64x64, more groups of 32 chains than SMs (p = 9728):
     # profiles/ising_ws_compact_L64_p9728.md
-    "ising_L64_compact": {"source": "8c638c33e6db10d8", "inst_per_attempt": 1.904,
-                          "shared_wavefronts_per_attempt": 0.365, "traffic_bytes_per_launch": 5169920},
-    # Ising 64x64, compact staging with the 16-bit table, three blocks per SM
-    # (p = 14592): profiles/ising_ws_t16_L64_p14592.md
-    "ising_L64_t16": {"source": "8c638c33e6db10d8", "inst_per_attempt": 1.989,
-                      "shared_wavefronts_per_attempt": 0.356, "traffic_bytes_per_launch": 7665664},
-    # 8-Potts 32x32 (p = 4096: 152 blocks of 27 chains): profiles/potts_ws_sweep_L32_p4096.md
-    "potts_L32": {"source": "8c638c33e6db10d8", "inst_per_attempt": 3.158, "shared_wavefronts_per_attempt": 0.582,
-                  "traffic_bytes_per_launch": 5122048},
+    "ising_L64_compact": {"source": "9d3df190ad49e213", "inst_per_attempt": 2.774, "shared_wavefronts_per_attempt": 0.357,
+                          "traffic_bytes_per_launch": 6343680},
+    # Ising 64x64, 16-bit table (p = 9824): profiles/ising_ws_t16_L64_p14592.md
+    "ising_L64_t16": {"source": "9d3df190ad49e213", "inst_per_attempt": 3.304, "shared_wavefronts_per_attempt": 0.336,
+                      "traffic_bytes_per_launch": 6523136},
+    # 8-Potts 32x32, p = 4096: profiles/potts_ws_sweep_L32_p4096.md
+    "potts_L32": {"source": "9d3df190ad49e213", "inst_per_attempt": 3.752, "shared_wavefronts_per_attempt": 0.558,
+                  "traffic_bytes_per_launch": 4323328},
 }
-# cycles per site of the Ising stream decider's loop run alone on one warp
-# (tests/gpu_decider_loop.cu, profiles/ising_decider_loop_replica.md)
-DECIDER_CYCLES_PER_ATTEMPT_ALONE = 36.6
-# the same for the 8-Potts slot decider (tests/gpu_potts_decider_loop.cu,
-# profiles/potts_decider_loop_replica.md)
-POTTS_DECIDER_CYCLES_PER_ATTEMPT_ALONE = 43.4
+# Cycles of one pass of a group alone on its SM (64 sites of an Ising row at L = 64, 32 of an
+# 8-Potts row at L = 32), weights of four iterations of 50 sweeps: the chain latency that
+# bounds a launch (profiles/ising_ws_sweep_L64_p1024.md, profiles/potts_ws_sweep_L32_p4096.md)
+PASS_CYCLES = 919.0
+PASS_SITES = 64
+POTTS_PASS_CYCLES = 832.0
+POTTS_PASS_SITES = 32
 # MUFU ex2 results per clock per SM (the special-function units: 4 per sub-partition
 # per clock); the FP32 reweighting evaluates one ex2 per contributing (beta, bin)
 MUFU_EX2_PER_CLK_PER_SM = 16
@@ -93,17 +91,6 @@ def sweep_source_sha16():
         text = re.sub(r"//[^\n]*", " ", text)
         h.update(" ".join(text.split()).encode())
     return h.hexdigest()[:16]
-
-
-def chains_per_block(p, n_sm):
-    """Chains per block of a warp-specialised sweep launch with the lattices staged in
-    shared memory: 32, or, while groups of 32 leave SMs idle, ceil(p / SMs)."""
-    return 32 if (p + 31) // 32 >= n_sm else (p + n_sm - 1) // n_sm
-
-
-def sweep_blocks(p, n_sm):
-    cpg = chains_per_block(p, n_sm)
-    return (p + cpg - 1) // cpg
 
 
 def counters(name):
@@ -381,13 +368,13 @@ def sweep_roofline(w, sweep_avg_ms, n_sm, sm_max):
     inst = c["inst_per_attempt"]
     achieved = inst * rate                                   # Gwarp-inst/s
     ok = c["matches_source"]
-    occupied = min(4 * n_sm, 4 * sweep_blocks(w["p"], n_sm))
-    latency = w["p"] * sm_max * 1e6 / DECIDER_CYCLES_PER_ATTEMPT_ALONE / 1e9
+    occupied = min(4 * n_sm, (w["p"] + 1) // 2)      # groups of two chains at L = 64
+    latency = w["p"] * PASS_SITES * sm_max * 1e6 / PASS_CYCLES / 1e9
     return {
         "bound": "alu", "achieved": achieved if ok else None, "peak": peak, "unit": "Gwarp-inst/s",
         "frac": achieved / peak if ok else None,
         "traffic": c["traffic_bytes_per_launch"] if ok else None,
-        "kernel": "ising_ws_kernel (weight-iteration sweeps, warp-specialised)",
+        "kernel": "sweep_kernel (weight-iteration sweeps: rows predicted, verified, repaired)",
         "launch_ms": sweep_avg_ms, "attempts_per_ns": rate,
         "warp_inst_per_attempt": inst, "counters_match_source": ok,
         "peak_note": "%d SMs x 4 schedulers x 1 warp-instruction/clock at %.0f MHz, of measured max clock"
@@ -396,8 +383,8 @@ def sweep_roofline(w, sweep_avg_ms, n_sm, sm_max):
         "frac_of_occupied_schedulers": achieved / (peak * occupied / (4 * n_sm)) if ok else None,
         # the three bounds on attempts/ns of the sweeps at the measured max clock: issue
         # (every scheduler busy at this instruction count), shared-memory LSU (one
-        # wavefront per clock per SM) and chain latency (p chains at the decider loop's
-        # cycles per attempt)
+        # wavefront per clock per SM) and chain latency (p chains at the cycles of a pass
+        # alone on its SM)
         "bounds_attempts_per_ns": {
             "issue": 4 * n_sm * sm_max * 1e6 / inst / 1e9,
             "lsu": n_sm * sm_max * 1e6 / c["shared_wavefronts_per_attempt"] / 1e9,
@@ -409,9 +396,7 @@ def sweep_roofline(w, sweep_avg_ms, n_sm, sm_max):
 
 def p_sweep(m, torch, stream, n_sm, sm_max):
     """Ising 64x64 weight-iteration launches at growing p: where the issue roofline
-    saturates.  One block of 32 chains per SM up to p = 32 x SMs; beyond, the compact
-    staging runs two blocks per SM, and three (the table of 16-bit threshold halves)
-    where that takes fewer waves: at 96 and 192 x SMs."""
+    saturates (one block of up to twelve groups of two chains per SM)."""
     timed = cuda_timer(torch, stream)
     peak = n_sm * 4 * sm_max * 1e6 / 1e9
     out = []
@@ -429,18 +414,12 @@ def p_sweep(m, torch, stream, n_sm, sm_max):
         c = counters("ising_L64_t16" if plan & m.MUCA_PLAN_TABLE16 else
                      "ising_L64_compact" if plan & m.MUCA_PLAN_COMPACT else "ising_L64")
         ok = c["matches_source"]
-        if "chains_per_block" in c:
-            # a warp issues for all 32 lanes: per attempt of a chain the counts scale
-            # with 1 / (chains per block) from the captured launch's
-            scale = c["chains_per_block"] / chains_per_block(p, n_sm)
-            c["inst_per_attempt"] *= scale
-            c["shared_wavefronts_per_attempt"] *= scale
         out.append({"p": p, "attempts_per_ns": rnd(rate), "compact": bool(plan & m.MUCA_PLAN_COMPACT),
-                    "blocks_per_sm": 3 if plan & m.MUCA_PLAN_TABLE16 else 2 if plan & m.MUCA_PLAN_COMPACT else 1,
+                    "table16": bool(plan & m.MUCA_PLAN_TABLE16),
                     "issue_frac": rnd(rate * c["inst_per_attempt"] / peak, 3) if ok else None,
                     "lsu_frac": rnd(rate * c["shared_wavefronts_per_attempt"] / (n_sm * sm_max * 1e-3), 3)
                     if ok else None,
-                    "latency_frac": rnd(rate / (p * sm_max * 1e-3 / DECIDER_CYCLES_PER_ATTEMPT_ALONE), 3)})
+                    "latency_frac": rnd(rate / (p * PASS_SITES * sm_max * 1e-3 / PASS_CYCLES), 3)})
     return out
 
 
@@ -520,12 +499,11 @@ def other_workloads(m, torch, stream, n_sm, sm_max):
                                    "frac": rnd(rate * c["inst_per_attempt"] / peak, 3) if c["matches_source"]
                                    else None,
                                    "counters_match_source": c["matches_source"],
-                                   "occupied_sms": min(n_sm, sweep_blocks(w["p"], n_sm)),
-                                   # p chains at the slot decider's cycles per attempt alone
+                                   # p chains at the cycles of a pass alone
                                    "latency_bound_attempts_per_ns": rnd(
-                                       w["p"] * sm_max * 1e-3 / POTTS_DECIDER_CYCLES_PER_ATTEMPT_ALONE),
+                                       w["p"] * POTTS_PASS_SITES * sm_max * 1e-3 / POTTS_PASS_CYCLES),
                                    "frac_of_latency_bound": rnd(
-                                       rate / (w["p"] * sm_max * 1e-3 / POTTS_DECIDER_CYCLES_PER_ATTEMPT_ALONE), 3)}
+                                       rate / (w["p"] * POTTS_PASS_SITES * sm_max * 1e-3 / POTTS_PASS_CYCLES), 3)}
             beta0 = workloads.ISING_BETA0 if w["model"] == workloads.ISING else workloads.POTTS8_BETA0
             lnw = workloads.canonical_lnw(w["model"], w["L"], w.get("fixed_beta", beta0))
             g.set_lnw(lnw - lnw.max())
@@ -699,10 +677,11 @@ def make_summary(r):
 
 
 def run_probe(args):
-    """One small launch of a workload's sweeps, for profiler captures: start, a 2-sweep
-    iteration and update (the launch skipped by -s 1), then one iteration of
-    --probe-sweeps sweeps (the captured launch); with --probe-phase produce, a 2-sweep
-    thermalisation (skipped) and production sweeps at the workload's weights."""
+    """One small launch of a workload's sweeps, for profiler captures: start, four
+    iterations of 50 sweeps with their updates (the launches skipped by -s 4), then one
+    iteration of --probe-sweeps sweeps (the captured launch); with --probe-phase produce,
+    a 2-sweep thermalisation (skipped by -s 1) and production sweeps at the workload's
+    weights."""
     import torch
     import paper_1212_3975_gb300 as m
     from paper_1212_3975_gb300 import build as b
@@ -717,8 +696,9 @@ def run_probe(args):
     if args.probe_phase == "produce":
         g.thermalize(2)          # at the workload's weights
     else:
-        g.iterate(2)
-        g.update_weights()
+        for _ in range(4):
+            g.iterate(50)
+            g.update_weights()
     torch.cuda.synchronize()
     t0 = time.perf_counter()
     if args.probe_phase == "produce":

@@ -75,7 +75,7 @@ extern "C" {
 typedef struct muca_config {
     int recursion;        /* MUCA_RECURSION_*; default accumulated */
     int correction_width; /* bins for the boundary slope (Sec. 3); 0 -> L */
-    int chains_per_block; /* multiple of 32, <= 256; 0 -> automatic */
+    int chains_per_block; /* multiple of 32, <= 256, or 0; the sweeps choose their own block shape */
     int staging;          /* MUCA_STAGING_*; 0 -> automatic */
     int ensemble;         /* MUCA_ENSEMBLE_*; 0 -> energy */
     double beta;          /* inverse temperature of the multimagnetic ensemble */
@@ -255,22 +255,25 @@ int muca_get_iteration(const muca_ctx *ctx); /* weight iterations done */
 
 /* How the sweep kernels stage this context's chains (introspection for tests and
  * tuning; the choice depends on L, p, the device and cfg->staging): a bit mask of
- *  MUCA_PLAN_LATTICE_SMEM   lattices in shared memory (else global memory, L1/L2),
+ *  MUCA_PLAN_LATTICE_SMEM   lattices in shared memory in launches with a histogram (else
+ *                           global memory, L1/L2; launches without a histogram stage
+ *                           them wherever they fit),
  *  MUCA_PLAN_HIST_SMEM      block histogram in shared memory (else global atomics),
  *  MUCA_PLAN_TABLE_SMEM     threshold table in shared memory (else global memory),
  *  MUCA_PLAN_PAIR_HIST      histogram of pairs of consecutive attempts,
- *  MUCA_PLAN_COMPACT        compact staging, two blocks per SM (more groups of 32
- *                           chains than SMs),
- *  MUCA_PLAN_WARP_SPECIALIZED  decider / producer / bookkeeper warps (L % 4 == 0),
+ *  MUCA_PLAN_COMPACT        compact staging (Ising, more groups of 32 chains than SMs):
+ *                           table and a histogram of single attempts in shared memory,
+ *                           lattices in global memory,
+ *  MUCA_PLAN_WARP_SPECIALIZED  deciding and drawing warps (always set),
  *  MUCA_PLAN_TABLE16        compact staging with the upper 16 bits of the thresholds
- *                           in shared memory, three blocks per SM (Ising, L % 32 == 0,
- *                           L >= 64, more than two groups of 32 chains per SM); a
- *                           draw whose upper half ties the table entry replays its
- *                           word from the 32-bit table, so results are unchanged,
+ *                           in shared memory (Ising, L = 64, two to two and a half
+ *                           groups of 32 chains per SM); a draw whose upper half ties
+ *                           the table entry reads the 32-bit table, so results are
+ *                           unchanged,
  *  MUCA_PLAN_HIST16         block histogram of 16-bit counts in shared memory, two bins
- *                           per word, added to the merged histogram every
- *                           floor(65535 / (32 L)) rows (Ising histograms too large for
- *                           32-bit counts in shared memory, e.g. 256 x 256).
+ *                           per word, added to the merged histogram before a count can
+ *                           overflow (Ising histograms too large for 32-bit counts in
+ *                           shared memory, e.g. 256 x 256).
  * Errors: MUCA_ERR_ARG (null context). */
 #define MUCA_PLAN_LATTICE_SMEM 1
 #define MUCA_PLAN_HIST_SMEM 2

@@ -3,7 +3,7 @@
 // of the whole iteration loop; plus a small timing-based autotuner.
 //
 // Every lattice is an ordinary context and follows exactly the trajectory it would
-// follow alone: the work units run the same warp-specialised bodies with the same
+// follow alone: the work units run the same sweep bodies with the same
 // arguments (seed, chain ids, iteration and sweep counters); only which SM runs a
 // unit, and when, differs.  The work queue is a monotone atomic counter, so no block
 // ever waits on another.
@@ -16,11 +16,14 @@
 #include <string>
 #include <vector>
 
-#include "ws_bodies.cuh"
+#include "sweep_small.cuh"
 
 namespace muca {
 namespace {
-using namespace ws;
+using namespace sweep;
+
+// groups of chains per work unit (and 2 warps each per block)
+constexpr int kBatchGroups = 4;
 
 struct BatchUnit {
     int job, cblk;
@@ -43,7 +46,6 @@ __device__ __forceinline__ SweepArgs batch_args(const BatchJob &j, int n_sweeps,
     a.q = j.q;
     a.p = j.p;
     a.p_pad = j.p_pad;
-    a.cpg = 32;
     a.row_words = j.row_words;
     a.lat_words = j.lat_words;
     a.n_bins = j.n_bins;
@@ -58,46 +60,55 @@ __device__ __forceinline__ SweepArgs batch_args(const BatchJob &j, int n_sweeps,
     return a;
 }
 
-// H: histogram mode (0 global, 1 shared per attempt, 2 shared per pair of attempts;
-// the Potts body without a bookkeeper warp counts per attempt)
-template <int MODEL, bool HIST, bool T, int H, bool Lt>
-__device__ __forceinline__ void body(const SweepArgs &a, int cblk, uint32_t *smem)
+// One work unit: the body of its lattice's shape (sweep_launch.cuh has the same cases,
+// with the histogram of pairs wherever the table is in shared memory).
+template <int MODEL, int LPC, bool ROW, int TAB, int HMODE>
+__device__ __forceinline__ void body(const SweepArgs &a, const BatchJob &j, int cblk, uint32_t *smem)
 {
-    if (MODEL == MUCA_ISING)
-        ising_ws_body<HIST, false, T, HIST ? H : 0, Lt>(a, cblk, smem);
-    else
-        potts_ws_body<HIST, false, T, (HIST && H) ? 1 : 0, Lt>(a, cblk, smem);
+    sweep_body<MODEL, LPC, ROW, true, TAB, HMODE>(a, cblk, kBatchGroups, j.lattice != 0, smem);
 }
 
 template <int MODEL, bool HIST>
-__device__ __forceinline__ void run_unit(const SweepArgs &a, int flags, int cblk, uint32_t *smem)
+__device__ __forceinline__ void run_unit(const SweepArgs &a, const BatchJob &j, int cblk, uint32_t *smem)
 {
-    if constexpr (MODEL == MUCA_ISING) {
-        if (flags & 8) {  // histogram of attempt pairs (table and lattices staged)
-            body<MODEL, HIST, true, 2, true>(a, cblk, smem);
-            return;
+    constexpr int HP = HIST ? kHistPairs : kHistNone, H1 = HIST ? kHistSingle : kHistNone;
+    constexpr int T16 = MODEL == MUCA_ISING ? kTabShared : kTabGlobal;
+    switch (j.lpc) {
+    case 1:
+        if constexpr (MODEL == MUCA_ISING) {
+            switch (a.L) {
+            case 4: small_body<4, HIST>(a, cblk, kBatchGroups, smem); break;
+            case 8: small_body<8, HIST>(a, cblk, kBatchGroups, smem); break;
+            case 12: small_body<12, HIST>(a, cblk, kBatchGroups, smem); break;
+            default: small_body<16, HIST>(a, cblk, kBatchGroups, smem);
+            }
         }
-    }
-    switch (flags & 7) {
-    case 0: body<MODEL, HIST, false, 0, false>(a, cblk, smem); break;
-    case 1: body<MODEL, HIST, false, 0, true>(a, cblk, smem); break;
-    case 2: body<MODEL, HIST, false, 1, false>(a, cblk, smem); break;
-    case 3: body<MODEL, HIST, false, 1, true>(a, cblk, smem); break;
-    case 4: body<MODEL, HIST, true, 0, false>(a, cblk, smem); break;
-    case 5: body<MODEL, HIST, true, 0, true>(a, cblk, smem); break;
-    case 6: body<MODEL, HIST, true, 1, false>(a, cblk, smem); break;
-    default: body<MODEL, HIST, true, 1, true>(a, cblk, smem); break;
+        break;
+    case 4:
+        if constexpr (MODEL == MUCA_POTTS) body<MODEL, 4, true, kTabShared, HP>(a, j, cblk, smem);
+        break;
+    case 8: body<MODEL, 8, true, kTabShared, HP>(a, j, cblk, smem); break;
+    case 16: body<MODEL, 16, true, T16, MODEL == MUCA_ISING ? HP : H1>(a, j, cblk, smem); break;
+    default:
+        if (j.row)
+            body<MODEL, 32, true, kTabGlobal, H1>(a, j, cblk, smem);
+        else if (!HIST || j.hist == kHistSingle)
+            body<MODEL, 32, false, kTabGlobal, H1>(a, j, cblk, smem);
+        else if (HIST && MODEL == MUCA_ISING && j.hist == kHist16)
+            body<MODEL, 32, false, kTabGlobal, HIST ? kHist16 : kHistNone>(a, j, cblk, smem);
+        else
+            body<MODEL, 32, false, kTabGlobal, HIST ? kHistGlobal : kHistNone>(a, j, cblk, smem);
     }
 }
 
 // Persistent sweep kernel of one weight iteration (or part of it); THERM: sweeps of
 // an intermediate thermalisation (no histogram).
 template <bool THERM>
-__global__ void __launch_bounds__(128, 1) batch_sweep_kernel(const BatchJob *jobs, const BatchUnit *units, int n_units,
+__global__ void __launch_bounds__(block_threads(kBatchGroups), 1) batch_sweep_kernel(const BatchJob *jobs, const BatchUnit *units, int n_units,
                                                           unsigned *queue, int n_sweeps, uint32_t sweep0)
 {
     extern __shared__ __align__(16) uint32_t smem[];
-    __shared__ int s_unit, s_model, s_flags, s_cblk;
+    __shared__ int s_unit, s_model, s_job, s_cblk;
     // The unit's arguments live in shared memory and the bodies read them where they
     // need them (the standalone kernels read theirs from the parameter bank); built in
     // registers they raised the register pressure of the bodies into spills.
@@ -111,7 +122,7 @@ __global__ void __launch_bounds__(128, 1) batch_sweep_kernel(const BatchJob *job
                 const BatchUnit un = units[u];
                 const BatchJob &j = jobs[un.job];
                 s_model = *j.active ? j.model : -1;  // -1: converged, frozen
-                s_flags = j.flags;
+                s_job = un.job;
                 s_cblk = un.cblk;
                 s_args = batch_args(j, n_sweeps, sweep0, THERM);
             }
@@ -120,9 +131,9 @@ __global__ void __launch_bounds__(128, 1) batch_sweep_kernel(const BatchJob *job
         if (s_unit >= n_units) break;
         const int model = s_model;
         if (model == MUCA_ISING)
-            run_unit<MUCA_ISING, !THERM>(s_args, s_flags, s_cblk, smem);
+            run_unit<MUCA_ISING, !THERM>(s_args, jobs[s_job], s_cblk, smem);
         else if (model == MUCA_POTTS)
-            run_unit<MUCA_POTTS, !THERM>(s_args, s_flags, s_cblk, smem);
+            run_unit<MUCA_POTTS, !THERM>(s_args, jobs[s_job], s_cblk, smem);
     }
 }
 
@@ -141,7 +152,7 @@ __global__ void batch_ktab_kernel(const BatchJob *jobs)
 {
     const BatchJob &j = jobs[blockIdx.y];
     if (!*j.active) return;
-    const int width = j.model == MUCA_ISING ? 5 : 9;
+    const int width = ktab_width(j.model);
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < j.n_bins * width; t += gridDim.x * blockDim.x) {
         const int b = t / width, k = t % width;
         uint32_t v;
@@ -243,25 +254,17 @@ int configure(muca_batch *b)
     b->smem = 0;
     b->max_bins = b->max_thr = b->max_ktab = 0;
     std::vector<std::pair<long long, BatchUnit>> units;
-    // Every block gets the shared memory of the largest job, so the histogram of
-    // attempt pairs is used only where it does not raise that maximum (more shared
-    // memory leaves less L1 to the jobs that read their tables from global memory).
-    size_t smem_plain = 0;
-    for (int i = 0; i < b->n_jobs; ++i) {
-        b->ctx[i]->cfg.staging = b->staging;
-        const SweepPlan pl = plan_sweeps(b->ctx[i], false, false);
-        smem_plain = std::max(smem_plain, pl.smem_bytes + ws_extra_smem(b->ctx[i]->model));
-    }
     for (int i = 0; i < b->n_jobs; ++i) {
         muca_ctx *c = b->ctx[i];
         c->cfg.staging = b->staging;
         if (c->cfg.ensemble != MUCA_ENSEMBLE_ENERGY)
             return fail(MUCA_ERR_ARG, "batched lattices need the energy ensemble (job " + std::to_string(i) + ")");
-        // pairs of attempts for Ising (its body has a bookkeeper warp here) within the
-        // shared memory of the largest job; the batched Potts body counts per attempt
-        SweepPlan pl = plan_sweeps(c, c->model == MUCA_ISING, false);
-        if (pl.hist_pairs && pl.smem_bytes + ws_extra_smem(c->model) > smem_plain) pl = plan_sweeps(c, false, false);
-        if (!pl.warp_specialized)
+        const SweepPlan pl = plan_sweeps(c, false, kBatchGroups);
+        const SweepShape shape = sweep_shape(c, pl, true, kBatchGroups);
+        // (pairs wherever the table is in shared memory: run_unit)
+        if (shape.groups != kBatchGroups || (shape.lpc > 1 && pl.hist_pairs != pl.table_smem))
+            return fail(MUCA_ERR_ARG, "batched staging exceeds shared memory");
+        if (c->L % 4 != 0)
             return fail(MUCA_ERR_ARG, "batched lattices need L % 4 == 0 (job " + std::to_string(i) + ")");
         BatchJob &j = b->h_jobs[i];
         j.model = c->model;
@@ -295,15 +298,21 @@ int configure(muca_batch *b)
         j.conv = b->d_conv + i;
         j.ctr3_therm = ((uint32_t)(c->seed >> 32) << 2) | kPhaseThermalize;
         j.therm = b->d_therm + i;
-        j.flags = (pl.hist_pairs ? 8 : 0) | (pl.table_smem ? 4 : 0) | (pl.hist_smem ? 2 : 0) | (pl.lattice_smem ? 1 : 0);
+        j.table_smem = pl.table_smem;
+        j.hist = hist_mode(pl);
+        j.lattice = shape.lattice;
+        j.lpc = shape.lpc;
+        j.row = shape.row;
         b->plan_flags[i] = plan_flags(pl);
-        b->smem = std::max(b->smem, pl.smem_bytes + ws_extra_smem(c->model));
+        b->smem = std::max(b->smem, shape.smem);
         b->max_bins = std::max(b->max_bins, c->n_bins);
         b->max_thr = std::max(b->max_thr, c->n_bins * c->n_de);
-        b->max_ktab = std::max(b->max_ktab, c->n_bins * (c->model == MUCA_ISING ? 5 : 9));
-        // cost of a unit ~ sites per sweep x time per site (Potts sites cost about 3 Ising sites)
-        const long long cost = (long long)c->V * (c->model == MUCA_ISING ? 1 : 3);
-        for (int cb = 0; cb < c->p_pad / 32; ++cb) units.push_back({cost, BatchUnit{i, cb}});
+        b->max_ktab = std::max(b->max_ktab, c->n_bins * ktab_width(c->model));
+        // cost of a unit ~ passes per sweep (a Potts pass takes about 1.3 Ising ones), or sites
+        const long long cost = shape.lpc == 1 ? (long long)c->V / 2
+                                              : (long long)c->L * (shape.row ? 1 : (c->L + 127) / 128) *
+                                                    (c->model == MUCA_ISING ? 10 : 13);
+        for (int cb = 0; cb < (c->p + shape.chains - 1) / shape.chains; ++cb) units.push_back({cost, BatchUnit{i, cb}});
     }
     std::stable_sort(units.begin(), units.end(),
                      [](const std::pair<long long, BatchUnit> &x, const std::pair<long long, BatchUnit> &y) {
@@ -347,7 +356,7 @@ int enqueue_iteration(muca_batch *b, int n_sweeps)
         } else {
             MUCA_CUDA_TRY(cudaMemsetAsync(b->d_queue, 0, sizeof(unsigned), b->stream));
         }
-        batch_sweep_kernel<false><<<b->grid, 128, b->smem, b->stream>>>(b->d_jobs, b->d_units, b->n_units, b->d_queue,
+        batch_sweep_kernel<false><<<b->grid, block_threads(kBatchGroups), b->smem, b->stream>>>(b->d_jobs, b->d_units, b->n_units, b->d_queue,
                                                                          s1 - s0, (uint32_t)s0);
         MUCA_CUDA_TRY(cudaGetLastError());
         note_launches(1);
@@ -462,10 +471,8 @@ int muca_batch_create(muca_batch **out, const muca_job *jobs, int n_jobs, const 
     }
     b->staging = cfg ? cfg->staging : MUCA_STAGING_AUTO;
     b->ctx.assign(n_jobs, nullptr);
-    // the persistent kernel's work units are groups of 32 chains
     muca_config jc{MUCA_RECURSION_ACCUMULATED, 0, 0, MUCA_STAGING_AUTO, MUCA_ENSEMBLE_ENERGY, 0.0};
     if (cfg) jc = *cfg;
-    if (jc.chains_per_block == 0) jc.chains_per_block = 32;
     b->cfg = jc;
     for (int i = 0; i < n_jobs; ++i) {
         int rc = muca_init(&b->ctx[i], jobs[i].model, jobs[i].L, jobs[i].q, jobs[i].p, jobs[i].seed, &jc, b->stream);
@@ -526,7 +533,7 @@ namespace {
 // of individual contexts, and the iteration counters of the random streams.
 int begin_iterations(muca_batch *b, int n_sweeps)
 {
-    // uint32 block histograms: 32 chains x sweeps x sites per launch below 2^31
+    // uint32 block histograms: at most 32 chains x sweeps x sites per launch below 2^31
     long long vmax = 0;
     for (muca_ctx *c : b->ctx) vmax = std::max<long long>(vmax, c->V);
     while (32LL * ((n_sweeps + b->split - 1) / b->split) * vmax >= (1LL << 31)) {
@@ -608,7 +615,7 @@ int enqueue_thermalization(muca_batch *b, int n_sweeps)
     for (int s = 0; s < split; ++s) {
         const int s0 = (int)((long long)n_sweeps * s / split), s1 = (int)((long long)n_sweeps * (s + 1) / split);
         MUCA_CUDA_TRY(cudaMemsetAsync(b->d_queue, 0, sizeof(unsigned), b->stream));
-        batch_sweep_kernel<true><<<b->grid, 128, b->smem, b->stream>>>(b->d_jobs, b->d_units, b->n_units, b->d_queue,
+        batch_sweep_kernel<true><<<b->grid, block_threads(kBatchGroups), b->smem, b->stream>>>(b->d_jobs, b->d_units, b->n_units, b->d_queue,
                                                                         s1 - s0, (uint32_t)s0);
         MUCA_CUDA_TRY(cudaGetLastError());
         note_launches(1);

@@ -257,21 +257,7 @@ int muca_init(muca_ctx **out, int model, int L, int q, int p, uint64_t seed, con
     }
     c->row_words = model == MUCA_ISING ? (L + 31) / 32 : (L + 3) / 4;
     c->lat_words = L * c->row_words;
-    // Fewer groups of 32 chains than SMs: the warp-specialised kernels (L % 4 == 0,
-    // energy ensemble, automatic block size) spread the chains over every SM, cpg per
-    // block.  A chain's attempts are sequential, so at small p the chains' own latency
-    // bounds the rate, and fewer chains per SM contend less for its shared memory.
-    // Only where the plan stages the lattices in shared memory: a block's chains then
-    // span part of a cache line of the chain-interleaved lattice, which in global
-    // memory costs more lines per warp access than it gains (8-Potts 128x128 at
-    // p = 4096: 35 attempts/ns spread against 70 with 32 chains per block).
-    c->cpg = 32;
     c->p_pad = (p + 31) / 32 * 32;
-    if (L % 4 == 0 && c0.ensemble == MUCA_ENSEMBLE_ENERGY && c0.chains_per_block == 0 && (p + 31) / 32 < c->n_sm &&
-        plan_sweeps(c).lattice_smem) {
-        c->cpg = (p + c->n_sm - 1) / c->n_sm;
-        c->p_pad = (p + c->cpg - 1) / c->cpg * 32;
-    }
     int rc = alloc_buffers(c);
     if (rc) {
         free_ctx(c);
@@ -647,9 +633,8 @@ struct CkptHeader {
     uint64_t lnw_version, samples_lnw_version;
 };
 
-// A device array in the file.  Per-chain arrays (rows x p_pad on the device: the
-// chain-interleaved layout, whose padding depends on the device's SM count) are
-// written as rows x p, so that a checkpoint loads on any device.
+// A device array in the file.  Per-chain arrays are written as rows x p: without the
+// padding chains, and the lattice (chain-major on the device) word by word.
 struct Blob {
     void *dev;
     size_t elem, rows;  // element bytes; rows of p_pad (per chain) or one row of `n`
@@ -673,6 +658,17 @@ std::vector<Blob> blobs(muca_ctx *c)
 }
 
 constexpr int32_t kCkptVersion = 3;
+
+// [rows][cols] 32-bit words to [cols][rows]
+void transpose_lattice(std::vector<uint8_t> &buf, size_t rows, size_t cols)
+{
+    std::vector<uint8_t> out(buf.size());
+    const uint32_t *in = reinterpret_cast<const uint32_t *>(buf.data());
+    uint32_t *o = reinterpret_cast<uint32_t *>(out.data());
+    for (size_t r = 0; r < rows; ++r)
+        for (size_t c = 0; c < cols; ++c) o[c * rows + r] = in[r * cols + c];
+    buf.swap(out);
+}
 
 // Spins of a checkpoint's lattice (rows x p words) are values of the model: Potts
 // bytes below q, and the bits / bytes past site L - 1 of a row's last word zero.
@@ -740,6 +736,7 @@ int muca_save(muca_ctx *ctx, const char *path)
         } else {
             // the p chains of every row, without the padding columns
             const size_t row = b.elem * (size_t)ctx->p;
+            if (b.dev == ctx->d_lat) transpose_lattice(buf, ctx->p_pad, ctx->lat_words);
             for (size_t r = 0; r < b.rows && ok; ++r)
                 ok = std::fwrite(buf.data() + r * b.elem * (size_t)ctx->p_pad, 1, row, f) == row;
         }
@@ -793,6 +790,7 @@ int muca_load(muca_ctx **out, const char *path, void *cuda_stream)
             const size_t row = b.elem * (size_t)ctx->p, drow = b.elem * (size_t)ctx->p_pad;
             dev.assign(drow * b.rows, 0);
             for (size_t r = 0; r < b.rows; ++r) std::memcpy(dev.data() + r * drow, buf.data() + r * row, row);
+            if (b.dev == ctx->d_lat) transpose_lattice(dev, ctx->lat_words, ctx->p_pad);
             if (cudaMemcpy(b.dev, dev.data(), dev.size(), cudaMemcpyHostToDevice) != cudaSuccess)
                 return bail(MUCA_ERR_CUDA, "checkpoint upload");
             chain_state[bi] = buf;

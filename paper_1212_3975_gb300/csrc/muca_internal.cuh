@@ -1,16 +1,13 @@
 // Internal declarations of libmuca (not part of the C ABI).
 //
-// Device data layout (chain-interleaved, so that the 32 chains of a warp touch 32
-// consecutive words at every step of their lockstep typewriter sweep):
+// Device data layout (chain-major, so that the lanes that share a chain read its rows
+// from consecutive bytes):
 //   Ising: one bit per site, bit j of word w of row y holds site x = 32 w + j
 //          (1 = spin +1); row_words = ceil(L / 32).
 //   Potts: one byte per site, byte j of word w of row y holds site x = 4 w + j;
 //          row_words = ceil(L / 4).
-//   word k = y * row_words + w of chain c lives at lat[k * p_pad + c].
-// The warp-specialised sweep kernels give each block a group of cpg <= 32 chains (fewer
-// than 32 when there are fewer than 32 chains per SM, so that every SM runs some):
-// p_pad = ceil(p / cpg) * 32, lanes beyond cpg work on padding columns past
-// ceil(p / cpg) * cpg, and padding chains are never read back.
+//   word k = y * row_words + w of chain c lives at lat[c * lat_words + k]; bits and bytes
+//   past a row's last site are zero.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -79,7 +76,7 @@ __host__ __device__ inline int n_de_of(int model) { return model == MUCA_ISING ?
 
 // Arguments of one sweep launch (plain values and device pointers).
 struct SweepArgs {
-    uint32_t *lat;        // [lat_words][p_pad]
+    uint32_t *lat;        // [p_pad][lat_words]
     int32_t *E;           // [p_pad] running energy
     int32_t *M;           // [p_pad] running magnetisation (Ising) / record scratch
     uint64_t *cnt;        // Potts packed state counts [2][p_pad]
@@ -90,7 +87,6 @@ struct SweepArgs {
     int32_t *M_rec;
     uint64_t *samples;    // [3][n_bins] production sums (n, sum|M|, sum M^2) or null
     int L, q, p, p_pad, row_words, lat_words, n_bins;
-    int cpg;              // chains per block of the warp-specialised bodies (<= 32)
     int n_sweeps;
     uint32_t sweep0;      // counter word 1 of the first sweep
     uint32_t iteration;   // counter word 2
@@ -99,17 +95,26 @@ struct SweepArgs {
     int rec_stride;       // records row stride (= p)
 };
 
-// staging flags of a sweep launch
+// staging of the sweep launches of a context
 struct SweepPlan {
-    bool table_smem, hist_smem, lattice_smem;
-    bool hist_pairs;        // warp-specialised: shared histogram of attempt pairs
-    bool warp_specialized;  // decider / producer / bookkeeper warps per 32 chains
-    bool compact;           // warp-specialised Ising: two blocks per SM (3-slot draw ring)
-    bool t16;               // compact with a table of 16-bit threshold halves: three blocks per SM
+    bool table_smem, hist_smem;
+    bool lattice_smem;      // of launches with a histogram (the others take what room it leaves)
+    bool hist_pairs;        // shared histogram of attempt pairs
+    bool compact;           // many chains: lattices in global memory, histogram of single attempts
+    bool t16;               // compact with a table of 16-bit threshold halves
     bool hist16;            // histogram of 16-bit counts, two bins per word, flushed by rows
-    int chains_per_block;
-    size_t smem_bytes;      // staging of the plan (table, histogram, lattices)
-    size_t table_bytes, hist_bytes, lat_bytes;  // its parts (0: not staged)
+    size_t smem_bytes;      // staging of the plan for 32 chains (table, histogram, lattices)
+    size_t table_bytes, hist_bytes;
+};
+
+// Shape of a sweep launch: lanes per chain, whether a row is one pass, groups (warps of
+// 32 / lpc chains) per block, lattices staged, shared memory.
+struct SweepShape {
+    int lpc;
+    bool row;
+    int groups, chains;  // per block
+    bool lattice;
+    size_t smem;
 };
 
 // Device view of one lattice of a batch (pointers into its context).
@@ -126,7 +131,8 @@ struct BatchJob {
     uint64_t *H;
     muca_iter_stats *stats;
     uint32_t *iteration;        // device counter of weight iterations (counter word 2)
-    int flags;                  // staging of the sweep body: 4 table, 2 histogram, 1 lattice in smem
+    int table_smem, hist, lattice;  // staging of the sweep body (sweep_body.cuh)
+    int lpc, row;               // lanes per chain; a row is one pass
     int *active;                // 0: the lattice is frozen (converged) and every batch kernel skips it
     int *conv;                  // iteration at which the lattice converged, -1 before
     uint32_t ctr3_therm;        // counter word 3 of thermalisation sweeps
@@ -142,7 +148,6 @@ struct muca_ctx {
     muca_config cfg;
     cudaStream_t stream;
     int device;
-    int cpg;                  // chains per group of the warp-specialised sweep kernels (<= 32)
     int n_sm;                 // streaming multiprocessors of the device (queried at init)
     int smem_per_sm;          // shared memory per SM and reserved per block (bytes, queried)
     int smem_reserved;
@@ -220,10 +225,16 @@ int launch_update(muca_ctx *ctx);
 int launch_stats(muca_ctx *ctx);
 int launch_reweight(muca_ctx *ctx, const double *d_betas, int n_beta, int precision,
                     double *const out[4] /* e, C, absm, chi: device [n_beta] each */);
-SweepPlan plan_sweeps(const muca_ctx *ctx, bool allow_pairs = true, bool allow_compact = true);
+constexpr int kMaxSmem = 227 * 1024;
+// groups per block: 0 for as many as suit p (a batch's blocks have a fixed number)
+SweepPlan plan_sweeps(const muca_ctx *ctx, bool allow_compact = true, int groups = 0);
+SweepShape sweep_shape(const muca_ctx *ctx, const SweepPlan &pl, bool hist, int groups = 0);
+int hist_mode(const SweepPlan &pl);
 int plan_flags(const SweepPlan &pl);  // MUCA_PLAN_* bit mask
 cudaError_t launch_batch_update(const BatchJob *d_jobs, int n_jobs, int max_thr, cudaStream_t st);
 int launch_ktab(muca_ctx *ctx);
+// kernel table: Ising [n_bins][5] by unequal neighbours, Potts [n_bins][9] by dE + 4
+__host__ __device__ constexpr int ktab_width(int model) { return model == MUCA_ISING ? 5 : 9; }
 // Scratch of the tiled reweighting kernels (reweight_kernels.cu): a per-bin part (five
 // FP64 arrays, a float copy of ln Omega, the sampled range) and a per-call part for
 // n_beta betas (tile parameters, shifts, item offsets, partial sums), 256-byte aligned
@@ -261,14 +272,19 @@ constexpr size_t kNoallocScratchBytes = rw_bin_part_bytes(kNoallocMaxBins) + rw_
 cudaError_t launch_reweight_buffers(double *scratch, const uint64_t *samples, const double *lnw, int model, int L,
                                     int q, const double *d_betas, int n_beta, int precision, double *d_out, int n_sm,
                                     cudaStream_t st);
-// shared memory of a warp-specialised launch beyond its staging, for launches with a
-// histogram and / or records (the defaults: the largest)
-size_t ws_extra_smem(int model, bool compact = false, bool hist = true, bool record = true);
 // multimagnetic Ising ensemble (muma.cu)
 int launch_muma_thresholds(muca_ctx *ctx);
 int launch_muma_sweeps(muca_ctx *ctx, uint32_t phase, int n_sweeps, uint32_t sweep0, uint32_t iteration, bool hist,
                        int32_t *E_rec, int32_t *M_rec);
-cudaError_t launch_ws_sweep(const SweepArgs &a, const SweepPlan &pl, int model, int blocks, bool hist, bool record,
-                            cudaStream_t st);
+// one sweep launch of either model (sweep_ising.cu, sweep_potts.cu)
+struct SweepLaunch {
+    const SweepArgs &args;
+    const SweepPlan &plan;
+    const SweepShape &shape;
+    int blocks;
+    cudaStream_t stream;
+};
+cudaError_t launch_sweep_ising(const SweepLaunch &l, bool hist);
+cudaError_t launch_sweep_potts(const SweepLaunch &l, bool hist);
 
 }  // namespace muca

@@ -56,9 +56,8 @@ __global__ void __launch_bounds__(128) muma_sweep_kernel(MumaArgs a)
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c < a.p) {
         const int L = a.L, V = L * L, RW = a.row_words;
-        uint32_t *lat = a.lat + c;
-        const size_t ps = (size_t)a.p_pad;
-        auto bit = [&](int x, int y) -> uint32_t { return (lat[(size_t)(y * RW + (x >> 5)) * ps] >> (x & 31)) & 1u; };
+        uint32_t *lat = a.lat + (size_t)c * (size_t)(L * RW);
+        auto bit = [&](int x, int y) -> uint32_t { return (lat[y * RW + (x >> 5)] >> (x & 31)) & 1u; };
         int E = a.E[c], M = a.M[c];
         for (int sw = 0; sw < a.n_sweeps; ++sw) {
             const uint32_t sweep = a.sweep0 + (uint32_t)sw;
@@ -74,7 +73,7 @@ __global__ void __launch_bounds__(128) muma_sweep_kernel(MumaArgs a)
                 const int b = (M + V) >> 1;
                 const uint32_t A = a.thr[b * 10 + (me ? 5 : 0) + unequal];
                 if (A == kAlways || u < A) {
-                    lat[(size_t)(y * RW + (x >> 5)) * ps] ^= 1u << (x & 31);
+                    lat[y * RW + (x >> 5)] ^= 1u << (x & 31);
                     E += 8 - 4 * unequal;
                     M -= me ? 2 : -2;
                 }

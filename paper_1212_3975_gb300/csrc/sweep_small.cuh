@@ -1,0 +1,268 @@
+// Ising sweep body of small lattices (L <= 16): one lane per chain, site by site.
+//
+// A pass of sweep_body.cuh takes a chain of some 600 cycles however few its sites, so on
+// rows of up to 16 sites deciding one site after the other is faster (three iterations of
+// 200 sweeps of 8 x 8 at p = 8, updates included: 2.05 ms with the earlier site-by-site
+// kernel, 2.60 with passes of a row, 1.73 with this body).  The dependent step is kept
+// short as follows: the table row of the next attempt is one of two candidates (this
+// attempt rejected or accepted), and both candidates' thresholds are loaded before this
+// attempt is decided, so a decision waits for one load and one select.
+//
+// A block has G groups of 32 chains: warps 0..G-1 decide, up to four more draw the random
+// numbers into a ring per group (16 sites per hand-off).  Every lane has a histogram of its
+// own, count of bin b at word 32 b + lane: the chains of a warp share a few bins, and
+// atomics on one address wait on each other, and the table loads on them.
+#pragma once
+#include "sweep_body.cuh"
+
+namespace muca {
+namespace sweep {
+
+constexpr int kSmallL = 16;
+
+// Draws of a chain: three hand-offs of 16 sites, then the first again so that no row
+// wraps; 4 mod 32 words from chain to chain (vector loads of a warp hit every bank).
+struct SmallRing {
+    static constexpr int kPhase = 16, kSites = 3 * kPhase, kStride = kSites + kPhase + 4;
+    static constexpr size_t kBytes = 32 * kStride * 4;
+};
+
+// shared memory of a launch: table, histograms (one per lane), lattices, rings
+__host__ __device__ constexpr size_t small_smem(int n_bins, int lat_words, int groups, bool hist)
+{
+    return (size_t)n_bins * 32 + ((hist ? (size_t)n_bins * 128 : 0) + (size_t)lat_words * 128 + SmallRing::kBytes) * groups;
+}
+
+// byte k of x, zero-extended / sign-extended
+__device__ __forceinline__ uint32_t ubyte(uint32_t x, int k)
+{
+    uint32_t d;
+    asm("prmt.b32 %0, %1, 0, %2;" : "=r"(d) : "r"(x), "r"(0x4440u | (uint32_t)k));
+    return d;
+}
+__device__ __forceinline__ uint32_t sbyte(uint32_t x, int k)
+{
+    uint32_t d;
+    asm("prmt.b32 %0, %1, 0, %2;" : "=r"(d) : "r"(x), "r"((uint32_t)k | (8u | (uint32_t)k) * 0x1110u));
+    return d;
+}
+
+// Table offsets 4 n and row changes 64 - 32 n of four sites, one per byte, for the
+// previous attempt rejected (0) / accepted (1); n = unequal neighbours.
+struct Quad {
+    uint32_t K0, K1, D0, D1;
+};
+__device__ __forceinline__ Quad quad_of(uint32_t lo, uint32_t hi, uint32_t q, int g)
+{
+    const uint32_t pre = 4u * spread4(lo >> (4 * g)) + 8u * spread4(hi >> (4 * g)), l = 4u * spread4(q >> (4 * g));
+    Quad r;
+    r.K0 = pre + l;
+    r.K1 = pre + 0x04040404u - l;
+    r.D0 = (0xC0C0C0C0u - 8u * r.K0) ^ 0x80808080u;  // (per byte 192 - 32 n >= 64: no borrow)
+    r.D1 = (0xC0C0C0C0u - 8u * r.K1) ^ 0x80808080u;
+    return r;
+}
+
+// L as a template parameter: the sites of a row are one unrolled block without branches.
+template <int L, bool HIST>
+__device__ __forceinline__ void small_body(const SweepArgs &a, const int cblk, const int G, uint32_t *smem)
+{
+    using Rg = SmallRing;
+    static_assert(L >= 4 && L <= kSmallL && L % 2 == 0, "small lattices");
+    constexpr int V = L * L, lat_words = L;
+    __syncthreads();  // (persistent kernel: smem may still be read by the previous unit)
+    const int tid = threadIdx.x, nt = block_threads(G), lane = tid & 31, warp = tid >> 5;
+    const int n_bins = a.n_bins, lw = 32 * G, c0 = cblk * lw;
+    uint32_t *const s_tab = smem;
+    uint32_t *const s_hist = s_tab + 8 * n_bins;          // [G][n_bins][32]
+    const int n_hist = HIST ? 32 * n_bins * G : 0;
+    uint32_t *const s_lat = s_hist + n_hist;              // [lat_words][lw]
+    uint32_t *const s_ring = s_lat + lat_words * lw;
+    for (int i = tid; i < 8 * n_bins; i += nt) s_tab[i] = (i & 7) < 5 ? a.ktab[5 * (i >> 3) + (i & 7)] : 0u;
+    for (int i = tid; i < n_hist; i += nt) s_hist[i] = 0u;
+    for (int i = tid; i < lat_words * lw; i += nt) {
+        const int k = i % lat_words, c = i / lat_words;
+        s_lat[k * lw + c] = c0 + c < a.p ? a.lat[(size_t)c0 * lat_words + i] : 0u;
+    }
+    __syncthreads();
+
+    const int phases = (int)(((long long)a.n_sweeps * V + Rg::kPhase - 1) / Rg::kPhase);
+    auto ring_of = [&](int grp) { return s_ring + grp * (int)(Rg::kBytes / 4) + lane * Rg::kStride; };
+
+    if (warp >= G) {
+        // ---------------- draws: a chain per lane, four sites per Philox block ------------------
+        const uint32_t quads = (uint32_t)V >> 2, key0 = a.key0, iter = a.iteration, ctr3 = a.ctr3;
+        uint32_t qd0 = 0u, ctr0 = a.sweep0;
+        int slot = 0;
+        for (int t = 0; t < phases; ++t) {
+            uint32_t qd = qd0, ctr1 = ctr0;
+            for (int grp = warp - G; grp < G; grp += draw_warps(G)) {
+                const uint32_t key1 = (uint32_t)(c0 + 32 * grp + lane);
+                // padding chains draw 2^32-1, which never accepts; the others at most
+                // 2^32-2, so that u < A decides
+                const bool active = key1 < (uint32_t)a.p;
+                uint32_t *const ring = ring_of(grp) + slot * Rg::kPhase;
+                qd = qd0;
+                ctr1 = ctr0;
+#pragma unroll
+                for (int pass = 0; pass < 4; ++pass) {
+                    uint4 b = philox4x32_10(make_uint4(qd, ctr1, iter, ctr3), key0, key1);
+                    b.x = active ? min(b.x, 0xFFFFFFFEu) : 0xFFFFFFFFu;
+                    b.y = active ? min(b.y, 0xFFFFFFFEu) : 0xFFFFFFFFu;
+                    b.z = active ? min(b.z, 0xFFFFFFFEu) : 0xFFFFFFFFu;
+                    b.w = active ? min(b.w, 0xFFFFFFFEu) : 0xFFFFFFFFu;
+                    *reinterpret_cast<uint4 *>(ring + 4 * pass) = b;
+                    if (slot == 0) *reinterpret_cast<uint4 *>(ring + 4 * pass + Rg::kSites) = b;
+                    if (++qd == quads) {
+                        qd = 0u;
+                        ++ctr1;
+                    }
+                }
+                bar_sync(1 + grp, 64);
+            }
+            qd0 = qd;
+            ctr0 = ctr1;
+            slot = slot == 2 ? 0 : slot + 1;
+        }
+    } else {
+        // ---------------- the chains ------------------------------------------------------------
+        const int grp = warp, c = c0 + 32 * grp + lane;
+        const bool active = c < a.p;
+        const uint32_t lat_s = (uint32_t)__cvta_generic_to_shared(s_lat + 32 * grp + lane), ls = 4u * (uint32_t)lw;
+        auto row_of = [&](int y) { return lds32(lat_s + (uint32_t)y * ls); };
+        const uint32_t tab0 = (uint32_t)__cvta_generic_to_shared(s_tab);
+        const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring_of(grp));
+        const bool record = !HIST && (a.E_rec || a.M_rec || a.samples);
+        // (count of the row at P: word 32 (P - tab0) / 32 + lane)
+        const uint32_t hist0 = (uint32_t)__cvta_generic_to_shared(s_hist + 32 * n_bins * grp + lane) - 4u * tab0;
+
+        // P0 / P1: table row before the site if the previous attempt was rejected / accepted
+        // (ap: which); D0 / D1: its change if the site accepts, A0 / A1: the thresholds
+        uint32_t P0 = tab0 + 32u * (uint32_t)(active ? (a.E[c] + 2 * V) >> 2 : V >> 1), P1 = P0;
+        bool ap = false;
+        uint32_t R = row_of(0), U = row_of(L - 1), D = row_of(1);
+        // unequal neighbours of a row's first site (its left one is site L - 1, old)
+        auto first_site = [&](uint32_t r, uint32_t u, uint32_t d) {
+            const uint32_t s = 0u - (r & 1u);  // (all bits: the spin)
+            return ((s ^ u) & 1u) + ((s ^ d) & 1u) + ((s ^ (r >> 1)) & 1u) + ((s ^ (r >> (L - 1))) & 1u);
+        };
+        const uint32_t n = first_site(R, U, D);
+        uint32_t D0 = 64u - 32u * n, D1 = D0;
+        uint32_t A0 = lds32(P0 + 4u * n), A1 = A0;
+        bar_sync(1 + grp, 64);
+        const int rows = a.n_sweeps * L;
+        int y = 0, sw = 0, pos = 0, lin = L, next_sync = Rg::kPhase;
+        int ups = 0;
+        for (int it = 0; it < rows; ++it) {
+            // the row's draws are handed off
+            if (lin > next_sync) {
+                if (next_sync < phases * Rg::kPhase) bar_sync(1 + grp, 64);
+                next_sync += Rg::kPhase;
+            }
+            const uint32_t us = ring_s + 4u * (uint32_t)pos;
+            uint32_t u[L];
+            if constexpr (L % 4 == 0) {
+#pragma unroll
+                for (int j = 0; j < L; j += 4)
+                    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                                 : "=r"(u[j]), "=r"(u[j + 1]), "=r"(u[j + 2]), "=r"(u[j + 3])
+                                 : "r"(us + 4u * j));
+            } else {
+#pragma unroll
+                for (int j = 0; j < L; j += 2)
+                    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(u[j]), "=r"(u[j + 1]) : "r"(us + 4u * j));
+            }
+            pos = pos + L >= Rg::kSites ? pos + L - Rg::kSites : pos + L;
+            lin += L;
+            const int y1 = y + 1 == L ? 0 : y + 1;
+            const uint32_t R1 = row_of(y1), D1w = row_of(y1 + 1 == L ? 0 : y1 + 1);
+            const uint32_t ua = R ^ U, ub = R ^ D, tr = R ^ (R >> 1), q = R ^ (R << 1);
+            const uint32_t lo = ua ^ ub ^ tr, hi = (ua & ub) | (tr & (ua ^ ub));
+            uint32_t Rw = R, last = 0u;  // last: unequal neighbours of the last site but its left one
+            Quad qd = quad_of(lo, hi, q, 0);
+#pragma unroll
+            for (int j = 0; j < L; ++j) {
+                // the next site's table offset and row change, for this attempt rejected / accepted
+                uint32_t K0, K1, E0, E1;
+                if (j + 1 == L) {
+                    // (of the row below only site 0 is needed yet: its upper neighbour is decided)
+                    const uint32_t n1 = first_site(R1, Rw, D1w);
+                    K0 = K1 = 4u * n1;
+                    E0 = E1 = 64u - 32u * n1;
+                } else if (j + 2 == L) {
+                    const uint32_t l = (q >> (L - 1)) & 1u;
+                    K0 = 4u * (last + l);
+                    K1 = 4u * (last + 1u - l);
+                    E0 = 64u - 8u * K0;
+                    E1 = 64u - 8u * K1;
+                } else {
+                    if ((j & 3) == 3) qd = quad_of(lo, hi, q, (j + 1) >> 2);
+                    const int k = (j + 1) & 3;
+                    K0 = ubyte(qd.K0, k);
+                    K1 = ubyte(qd.K1, k);
+                    E0 = sbyte(qd.D0, k);
+                    E1 = sbyte(qd.D1, k);
+                }
+                const uint32_t Pc = ap ? P1 : P0, Pa = Pc + (ap ? D1 : D0);
+                const uint32_t B0 = lds32(Pc + K0), B1 = lds32(Pa + K1);
+                const bool acc = u[j] < (ap ? A1 : A0);
+                if (HIST) red_shared(hist0 + 4u * (acc ? Pa : Pc), 1u);
+                Rw ^= acc ? 1u << j : 0u;
+                if (j == 0)  // the row's last site sees the updated site 0 to its right
+                    last = ((ua >> (L - 1)) & 1u) + ((ub >> (L - 1)) & 1u) + (((R >> (L - 1)) ^ Rw) & 1u);
+                P0 = Pc;
+                P1 = Pa;
+                D0 = E0;
+                D1 = E1;
+                A0 = B0;
+                A1 = B1;
+                ap = acc;
+            }
+            asm volatile("st.shared.u32 [%0], %1;" ::"r"(lat_s + (uint32_t)y * ls), "r"(Rw) : "memory");
+            ups += __popc(Rw);
+            if (y1 == 0) {
+                if (record && active) {
+                    const int b = (int)(((ap ? P1 : P0) - tab0) >> 5), M = 2 * ups - V;
+                    if (a.E_rec) a.E_rec[(size_t)sw * a.rec_stride + c] = 4 * b - 2 * V;
+                    if (a.M_rec) a.M_rec[(size_t)sw * a.rec_stride + c] = M;
+                    if (a.samples) {
+                        const unsigned long long am = (unsigned long long)(M < 0 ? -M : M);
+                        unsigned long long *sp = reinterpret_cast<unsigned long long *>(a.samples);
+                        atomicAdd(&sp[b], 1ull);
+                        atomicAdd(&sp[n_bins + b], am);
+                        atomicAdd(&sp[2 * n_bins + b], am * am);
+                    }
+                }
+                ++sw;
+                if (it + 1 < rows) ups = 0;
+            }
+            // (R1 and D1w were read before this row was stored: at L >= 4 they are other rows)
+            U = Rw;
+            R = R1;
+            D = D1w;
+            y = y1;
+        }
+        if (active) {
+            a.E[c] = 4 * (int)(((ap ? P1 : P0) - tab0) >> 5) - 2 * V;
+            a.M[c] = 2 * ups - V;
+        }
+    }
+    __syncthreads();
+    for (int i = tid; i < lat_words * lw; i += nt) {
+        const int k = i % lat_words, c = i / lat_words;
+        if (c0 + c < a.p) a.lat[(size_t)c0 * lat_words + i] = s_lat[k * lw + c];
+    }
+    if (HIST) {
+        // a warp per bin: counts of the block's chains (padding chains left out)
+        for (int b = warp; b < n_bins; b += nt >> 5) {
+            uint32_t x = 0u;
+            for (int g = 0; g < G; ++g)
+                if (c0 + 32 * g + lane < a.p) x += s_hist[32 * (n_bins * g + b) + lane];
+            x = __reduce_add_sync(~0u, x);
+            if (lane == 0 && x) atomicAdd(reinterpret_cast<unsigned long long *>(a.H + b), (unsigned long long)x);
+        }
+    }
+}
+
+}  // namespace sweep
+}  // namespace muca

@@ -42,13 +42,13 @@ __global__ void thresholds_kernel(const double *lnw, const uint8_t *acc, uint32_
     thr[t] = A;
 }
 
-// Kernel layout of the thresholds for the warp-specialised sweep bodies: one row per
+// Kernel layout of the thresholds for the sweep bodies: one row per
 // bin, one column per local configuration so that the column offset follows from the
 // neighbours without a branch.  Ising: column = number of unequal neighbours n
 // (dE = 8 - 4n, so n = 2 is dE = 0 and always accepts); Potts: column = dE + 4.
 __global__ void ktab_kernel(const uint32_t *thr, uint32_t *ktab, int model, int n_bins)
 {
-    const int width = model == MUCA_ISING ? 5 : 9;
+    const int width = ktab_width(model);
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n_bins * width) return;
     const int b = t / width, k = t % width;
@@ -302,7 +302,7 @@ int launch_update(muca_ctx *ctx)
 
 int launch_ktab(muca_ctx *ctx)
 {
-    const int width = ctx->model == MUCA_ISING ? 5 : 9;
+    const int width = ktab_width(ctx->model);
     const int n = ctx->n_bins * width;
     ktab_kernel<<<(n + 255) / 256, 256, 0, ctx->stream>>>(ctx->d_thr, ctx->d_ktab, ctx->model, ctx->n_bins);
     MUCA_CUDA_TRY(cudaGetLastError());
