@@ -361,7 +361,7 @@ int enqueue_iteration(muca_batch *b, int n_sweeps)
         MUCA_CUDA_TRY(cudaGetLastError());
         note_launches(1);
     }
-    cudaError_t e = launch_batch_update(b->d_jobs, b->n_jobs, b->max_thr, b->stream);
+    cudaError_t e = launch_batch_update(b->d_jobs, b->n_jobs, b->max_bins, b->max_thr, b->stream);
     if (e != cudaSuccess) return cuda_fail(e, "batched weight update");
     dim3 g((b->max_ktab + 255) / 256, b->n_jobs);
     batch_ktab_kernel<<<g, 256, 0, b->stream>>>(b->d_jobs);
@@ -590,7 +590,7 @@ int muca_batch_iterate(muca_batch *b, int n_iterations, int n_sweeps, int use_gr
             b->g_sweeps = n_sweeps;
         }
         MUCA_CUDA_TRY(cudaGraphLaunch(b->gexec, b->stream));
-        note_launches((uint64_t)n_iterations * (4 + b->split));
+        note_launches((uint64_t)n_iterations * (5 + b->split));
     } else {
         for (int i = 0; i < n_iterations; ++i) {
             int rc = enqueue_iteration(b, n_sweeps);

@@ -231,7 +231,7 @@ SweepPlan plan_sweeps(const muca_ctx *ctx, bool allow_compact = true, int groups
 SweepShape sweep_shape(const muca_ctx *ctx, const SweepPlan &pl, bool hist, int groups = 0);
 int hist_mode(const SweepPlan &pl);
 int plan_flags(const SweepPlan &pl);  // MUCA_PLAN_* bit mask
-cudaError_t launch_batch_update(const BatchJob *d_jobs, int n_jobs, int max_thr, cudaStream_t st);
+cudaError_t launch_batch_update(const BatchJob *d_jobs, int n_jobs, int max_bins, int max_thr, cudaStream_t st);
 int launch_ktab(muca_ctx *ctx);
 // kernel table: Ising [n_bins][5] by unequal neighbours, Potts [n_bins][9] by dE + 4
 __host__ __device__ constexpr int ktab_width(int model) { return model == MUCA_ISING ? 5 : 9; }

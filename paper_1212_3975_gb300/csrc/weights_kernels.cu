@@ -68,16 +68,131 @@ struct BlockStats {
     int lo, hi;
 };
 
-// Single-block update (blockDim.x = 1024):
+// The update runs as two kernels.  The recursion's differences (two logarithms and two
+// divisions in FP64 per bin, at two FP64 operations per clock and SM: 0.15 ms for 4097
+// bins on one SM) take a grid of blocks; what follows is one block per lattice
+// (blockDim.x = 1024):
 //   1. convergence statistics of H over accessible bins (Sec. 3);
-//   2. recursion (Sec. 2) into per-pair differences d[u] (accumulated) or values;
-//   3. sequential prefix over accessible bins in ascending order (thread 0);
-//   4. boundary correction beyond [lo, hi] with the slope of the innermost
+//   2. prefix sums of the differences over accessible bins in ascending order, rounded
+//      as the sequential sum (prefix_piece);
+//   3. boundary correction beyond [lo, hi] with the slope of the innermost
 //      `width` bins (Sec. 3);
-//   5. ln W -= max over accessible bins; inaccessible bins = 0.
-__device__ __forceinline__ void update_body(double *lnw, double *P, double *scratch, const uint64_t *H,
-                                            const uint8_t *acc, int n_bins, int accumulated, int width_cfg,
-                                            muca_iter_stats *stats)
+//   4. ln W -= max over accessible bins; inaccessible bins = 0.
+constexpr int kPiece = 4096;  // bins of the prefix staged at a time
+
+// Sequential FP64 sum cur += x[i] of n values in shared memory, in place, by one warp, 128
+// values at a time; returns the last sum.  The result is that of adding one value after
+// the other, bit for bit: while the sum stays in one binade it is a multiple k of one unit
+// u in the last place, and adding x rounds to k + (x / u rounded to the nearest integer),
+// so a run of additions is a prefix sum of integers.  Where that does not hold (a sum that
+// leaves the binade or changes sign, an x / u halfway between integers, an x above the
+// binade, a sum of zero) the one addition is done in FP64.  A chain of FP64 additions takes
+// 117 cycles per value on this GPU (two FP64 operations per clock and SM): 0.23 ms for the
+// 4097 bins of a 64 x 64 Ising lattice, 0.93 ms for 128 x 128, against 0.01 ms and 0.04 ms.
+__device__ __forceinline__ double prefix_piece(double *x, int n, double cur, int lane)
+{
+    constexpr unsigned long long one = 1ull << 52, frac = one - 1ull;
+    for (int i = 0; i < n;) {
+        const unsigned long long cb = (unsigned long long)__double_as_longlong(cur);
+        const int ce = (int)(cb >> 52) & 0x7FF;
+        const long long mag = (long long)((cb & frac) | one), k = cb >> 63 ? -mag : mag;
+        const bool zero = cb == 0ull, regular = ce > 0 && ce < 0x7FF;
+        long long v[4];   // the lane's inclusive sums of rounded integers
+        int good = 4;     // values of the lane before the first that needs FP64
+        long long sum = 0;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const int j = i + 4 * lane + t;
+            bool ok = j < n && (regular || zero);
+            if (ok) {
+                const unsigned long long b = (unsigned long long)__double_as_longlong(x[j]);
+                if (zero) {
+                    ok = (b << 1) == 0ull;
+                } else {
+                    int e = (int)(b >> 52) & 0x7FF;
+                    const unsigned long long mt = (b & frac) | (e ? one : 0ull);
+                    const int sh = ce - (e ? e : 1);
+                    ok = e != 0x7FF && sh >= 0;
+                    if (ok && sh <= 54) {
+                        const unsigned long long half = sh ? 1ull << (sh - 1) : 0ull;
+                        const unsigned long long low = sh ? mt & ((half << 1) - 1ull) : 0ull;
+                        ok = !(sh && low == half);
+                        const long long r = (long long)((mt + half) >> sh);
+                        sum += b >> 63 ? -r : r;
+                    }
+                }
+            }
+            v[t] = sum;
+            if (!ok) good = min(good, t);
+        }
+        long long incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long y = __shfl_up_sync(~0u, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const long long below = k + incl - sum;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            v[t] += below;
+            const unsigned long long q = (unsigned long long)(v[t] < 0 ? -v[t] : v[t]);
+            if (!zero && !(q > one && q < one << 1 && (v[t] < 0) == (k < 0))) good = min(good, t);
+        }
+        const unsigned stop = __ballot_sync(~0u, good < 4);
+        const int first = stop ? __ffs(stop) - 1 : 32;
+        const int done = stop ? 4 * first + __shfl_sync(~0u, good, first & 31) : 128;  // (values past n stop it)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            if (4 * lane + t < done) {
+                const unsigned long long q = (unsigned long long)(v[t] < 0 ? -v[t] : v[t]);
+                const unsigned long long bits = zero ? 0ull : (q & frac) | (unsigned long long)ce << 52 | (cb & (1ull << 63));
+                x[i + 4 * lane + t] = __longlong_as_double((long long)bits);
+            }
+        }
+        __syncwarp();
+        if (done > 0) cur = x[i + done - 1];
+        i += done;
+        if (done < 128 && i < n) {
+            cur = __dadd_rn(cur, x[i]);
+            __syncwarp();
+            if (lane == 0) x[i] = cur;
+            ++i;
+        }
+        __syncwarp();
+    }
+    return cur;
+}
+
+// Recursion (Sec. 2) of bin u: scratch[v] = difference to bin v from the accessible bin u
+// before it (accumulated form), or ln W after the simple recursion.
+__device__ __forceinline__ void update_bin(const double *lnw, double *P, double *scratch, const uint64_t *H,
+                                           const uint8_t *acc, int n_bins, int accumulated, int u)
+{
+    if (!acc[u]) return;
+    if (accumulated) {
+        int v = u + 1;
+        while (v < n_bins && !acc[v]) ++v;
+        if (v >= n_bins) return;
+        double d = __dsub_rn(lnw[v], lnw[u]);
+        const uint64_t hu_i = H[u], hv_i = H[v];
+        if (hu_i > 0 && hv_i > 0) {
+            const double hu = (double)hu_i, hv = (double)hv_i;
+            const double g0 = __ddiv_rn(__dmul_rn(hu, hv), __dadd_rn(hu, hv));
+            const double pu = __dadd_rn(P[u], g0);
+            P[u] = pu;
+            const double g = __ddiv_rn(g0, pu);
+            d = __dsub_rn(d, __dmul_rn(g, __dsub_rn(log(hv), log(hu))));
+        }
+        scratch[v] = d;
+    } else {
+        double v = lnw[u];
+        if (H[u] > 0) v = __dsub_rn(v, log((double)H[u]));
+        scratch[u] = v;
+    }
+}
+
+__device__ __forceinline__ void update_body(double *lnw, const double *scratch, const uint64_t *H, const uint8_t *acc,
+                                            int n_bins, int accumulated, int width_cfg, muca_iter_stats *stats)
 {
     __shared__ unsigned long long s_total[32], s_min[32], s_max[32], s_ns[32], s_K[32];
     __shared__ int s_lo[32], s_hi[32];
@@ -136,57 +251,36 @@ __device__ __forceinline__ void update_body(double *lnw, double *P, double *scra
     }
     __syncthreads();
 
-    // 2. recursion.  scratch[u] = difference to the next accessible bin (accumulated)
+    // 2. prefix in ascending order
     if (accumulated) {
-        for (int u = tid; u < n_bins; u += blockDim.x) {
-            if (!acc[u]) continue;
-            int v = u + 1;
-            while (v < n_bins && !acc[v]) ++v;
-            if (v >= n_bins) continue;
-            double d = __dsub_rn(lnw[v], lnw[u]);
-            const uint64_t hu_i = H[u], hv_i = H[v];
-            if (hu_i > 0 && hv_i > 0) {
-                const double hu = (double)hu_i, hv = (double)hv_i;
-                const double g0 = __ddiv_rn(__dmul_rn(hu, hv), __dadd_rn(hu, hv));
-                const double pu = __dadd_rn(P[u], g0);
-                P[u] = pu;
-                const double g = __ddiv_rn(g0, pu);
-                d = __dsub_rn(d, __dmul_rn(g, __dsub_rn(log(hv), log(hu))));
-            }
-            scratch[u] = d;
-        }
-    } else {
-        for (int b = tid; b < n_bins; b += blockDim.x) {
-            if (!acc[b]) continue;
-            double v = lnw[b];
-            if (H[b] > 0) v = __dsub_rn(v, log((double)H[b]));
-            scratch[b] = v;
-        }
-    }
-    __syncthreads();
-
-    // 3. prefix in ascending order (one thread: keeps the oracle's rounding order)
-    if (tid == 0) {
-        if (accumulated) {
+        __shared__ double s_d[kPiece];
+        __shared__ int s_first;
+        if (tid == 0) {
             int u = 0;
             while (!acc[u]) ++u;
-            double cur = 0.0;
-            lnw[u] = cur;
-            for (int v = u + 1; v < n_bins; ++v) {
-                if (!acc[v]) continue;
-                cur = __dadd_rn(cur, scratch[u]);
-                lnw[v] = cur;
-                u = v;
-            }
+            s_first = u;
         }
-    }
-    if (!accumulated) {
+        double cur = 0.0;  // (warp 0)
+        for (int b0 = 0; b0 < n_bins; b0 += kPiece) {
+            const int n = min(kPiece, n_bins - b0);
+            __syncthreads();
+            // (an inaccessible bin adds nothing; the first accessible one has no difference)
+            for (int i = tid; i < n; i += blockDim.x)
+                s_d[i] = acc[b0 + i] && b0 + i != s_first ? scratch[b0 + i] : 0.0;
+            __syncthreads();
+            if (warp == 0) cur = prefix_piece(s_d, n, cur, lane);
+            __syncthreads();
+            for (int i = tid; i < n; i += blockDim.x)
+                if (acc[b0 + i]) lnw[b0 + i] = s_d[i];
+            __syncthreads();
+        }
+    } else {
         for (int b = tid; b < n_bins; b += blockDim.x)
             if (acc[b]) lnw[b] = scratch[b];
     }
     __syncthreads();
 
-    // 4. boundary correction
+    // 3. boundary correction
     const int slo = sh_lo, shi = sh_hi;
     if (slo >= 0 && shi > slo) {
         const int width = min(width_cfg, shi - slo);
@@ -210,7 +304,7 @@ __device__ __forceinline__ void update_body(double *lnw, double *P, double *scra
     }
     __syncthreads();
 
-    // 5. normalisation: max over accessible bins is 0
+    // 4. normalisation: max over accessible bins is 0
     double top = -INFINITY;
     for (int b = tid; b < n_bins; b += blockDim.x)
         if (acc[b]) top = fmax(top, lnw[b]);
@@ -226,19 +320,34 @@ __device__ __forceinline__ void update_body(double *lnw, double *P, double *scra
     for (int b = tid; b < n_bins; b += blockDim.x) lnw[b] = acc[b] ? __dsub_rn(lnw[b], top) : 0.0;
 }
 
-__global__ void __launch_bounds__(1024) update_kernel(double *lnw, double *P, double *scratch, const uint64_t *H,
-                                                      const uint8_t *acc, int n_bins, int accumulated,
-                                                      int width_cfg, muca_iter_stats *stats)
+__global__ void update_bins_kernel(const double *lnw, double *P, double *scratch, const uint64_t *H, const uint8_t *acc,
+                                   int n_bins, int accumulated)
 {
-    update_body(lnw, P, scratch, H, acc, n_bins, accumulated, width_cfg, stats);
+    const int u = blockIdx.x * blockDim.x + threadIdx.x;
+    if (u < n_bins) update_bin(lnw, P, scratch, H, acc, n_bins, accumulated, u);
 }
 
-// one block per lattice of a batch
+__global__ void __launch_bounds__(1024) update_kernel(double *lnw, const double *scratch, const uint64_t *H,
+                                                      const uint8_t *acc, int n_bins, int accumulated, int width_cfg,
+                                                      muca_iter_stats *stats)
+{
+    update_body(lnw, scratch, H, acc, n_bins, accumulated, width_cfg, stats);
+}
+
+// bins of every lattice of a batch (blockIdx.y = lattice), then one block per lattice
+__global__ void update_bins_batch_kernel(const BatchJob *jobs)
+{
+    const BatchJob &j = jobs[blockIdx.y];
+    if (!*j.active) return;  // converged lattice: frozen
+    const int u = blockIdx.x * blockDim.x + threadIdx.x;
+    if (u < j.n_bins) update_bin(j.lnw, j.P, j.wscratch, j.H, j.acc, j.n_bins, j.accumulated, u);
+}
+
 __global__ void __launch_bounds__(1024) update_batch_kernel(const BatchJob *jobs)
 {
     const BatchJob &j = jobs[blockIdx.x];
-    if (!*j.active) return;  // converged lattice: frozen
-    update_body(j.lnw, j.P, j.wscratch, j.H, j.acc, j.n_bins, j.accumulated, j.width, j.stats);
+    if (!*j.active) return;
+    update_body(j.lnw, j.wscratch, j.H, j.acc, j.n_bins, j.accumulated, j.width, j.stats);
 }
 
 // thresholds of every lattice of a batch: blockIdx.y = lattice
@@ -265,15 +374,18 @@ __global__ void thresholds_batch_kernel(const BatchJob *jobs)
 
 }  // namespace
 
-cudaError_t launch_batch_update(const BatchJob *d_jobs, int n_jobs, int max_thr, cudaStream_t st)
+cudaError_t launch_batch_update(const BatchJob *d_jobs, int n_jobs, int max_bins, int max_thr, cudaStream_t st)
 {
-    update_batch_kernel<<<n_jobs, 1024, 0, st>>>(d_jobs);
+    update_bins_batch_kernel<<<dim3((max_bins + 127) / 128, n_jobs), 128, 0, st>>>(d_jobs);
     cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    update_batch_kernel<<<n_jobs, 1024, 0, st>>>(d_jobs);
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     dim3 grid((max_thr + 255) / 256, n_jobs);
     thresholds_batch_kernel<<<grid, 256, 0, st>>>(d_jobs);
     e = cudaGetLastError();
-    if (e == cudaSuccess) note_launches(2);
+    if (e == cudaSuccess) note_launches(3);
     return e;
 }
 
@@ -292,11 +404,14 @@ int launch_thresholds(muca_ctx *ctx)
 int launch_update(muca_ctx *ctx)
 {
     const int width = ctx->cfg.correction_width > 0 ? ctx->cfg.correction_width : ctx->L;
-    update_kernel<<<1, 1024, 0, ctx->stream>>>(ctx->d_lnw, ctx->d_P, ctx->d_wscratch, ctx->d_H, ctx->d_acc, ctx->n_bins,
-                                               ctx->cfg.recursion == MUCA_RECURSION_ACCUMULATED, width,
-                                               ctx->d_stats);
+    const int accumulated = ctx->cfg.recursion == MUCA_RECURSION_ACCUMULATED;
+    update_bins_kernel<<<(ctx->n_bins + 127) / 128, 128, 0, ctx->stream>>>(ctx->d_lnw, ctx->d_P, ctx->d_wscratch, ctx->d_H,
+                                                                          ctx->d_acc, ctx->n_bins, accumulated);
     MUCA_CUDA_TRY(cudaGetLastError());
-    note_launches(1);
+    update_kernel<<<1, 1024, 0, ctx->stream>>>(ctx->d_lnw, ctx->d_wscratch, ctx->d_H, ctx->d_acc, ctx->n_bins, accumulated,
+                                               width, ctx->d_stats);
+    MUCA_CUDA_TRY(cudaGetLastError());
+    note_launches(2);
     return launch_thresholds(ctx);
 }
 
