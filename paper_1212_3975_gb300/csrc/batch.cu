@@ -38,6 +38,7 @@ __device__ __forceinline__ SweepArgs batch_args(const BatchJob &j, int n_sweeps,
     a.cnt = j.cnt;
     a.thr = j.thr;
     a.ktab = j.ktab;
+    a.ktab31 = j.ktab + (size_t)j.n_bins * ktab_width(j.model);
     a.H = j.H;
     a.E_rec = nullptr;
     a.M_rec = nullptr;
@@ -163,6 +164,7 @@ __global__ void batch_ktab_kernel(const BatchJob *jobs)
             v = dE == 0 ? kAlways : j.thr[b * 8 + (dE < 0 ? dE + 4 : dE + 3)];
         }
         j.ktab[t] = v;
+        j.ktab[j.n_bins * width + t] = v >> 1;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) *j.iteration += 1u;
 }

@@ -152,7 +152,7 @@ int alloc_buffers(muca_ctx *c)
     if ((rc = dalloc(&c->d_wscratch, nb, "update scratch"))) return rc;
     if ((rc = dalloc(&c->d_acc, nb, "accessible bins"))) return rc;
     if ((rc = dalloc(&c->d_thr, nb * c->n_de, "thresholds"))) return rc;
-    if ((rc = dalloc(&c->d_ktab, nb * 9, "kernel thresholds"))) return rc;
+    if ((rc = dalloc(&c->d_ktab, 2 * nb * ktab_width(c->model), "kernel thresholds"))) return rc;
     if ((rc = dalloc(&c->d_H, nb, "histogram"))) return rc;
     if ((rc = dalloc(&c->d_samples, 3 * nb, "production sums"))) return rc;
     if ((rc = dalloc(&c->d_stats, 1, "stats"))) return rc;

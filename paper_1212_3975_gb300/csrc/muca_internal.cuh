@@ -82,6 +82,7 @@ struct SweepArgs {
     uint64_t *cnt;        // Potts packed state counts [2][p_pad]
     const uint32_t *thr;  // [n_bins][n_de]
     const uint32_t *ktab; // kernel table: Ising [n_bins][5] by unequal neighbours, Potts [n_bins][9] by dE+4
+    const uint32_t *ktab31; // the same, entries >> 1
     uint64_t *H;          // merged histogram [n_bins] (uint64, atomically added)
     int32_t *E_rec;       // [n_sweeps][rec_stride] or null
     int32_t *M_rec;

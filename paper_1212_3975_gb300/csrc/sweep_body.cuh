@@ -27,11 +27,16 @@
 // A lane holds four consecutive sites, one per byte; a chain takes LPC lanes (4 LPC sites
 // per pass), a warp (a group) 32 / LPC chains.  A lane composes the one-bit maps of its
 // sites for both values of the incoming bit; two ballots and a prefix over the ballots'
-// bits carry the decisions from lane to lane, and a shuffle scan the bin changes.  A pass
-// is a chain of about 350 cycles whatever its sites, so a row in one pass (ROW, L <= 4 LPC)
-// is what shortens a sweep.  A block has G groups: warps 0..G-1 decide, warp G + i draws
-// the random numbers of group i (Philox) into a ring, 16 LPC sites per hand-off (one
-// named barrier per group).
+// bits carry the decisions from lane to lane, and bytes in shared memory the bin changes.
+// A pass is a chain of dependent steps whatever its sites, so a row in one pass (ROW,
+// L <= 4 LPC) is what shortens a sweep.  A block has G groups: warps 0..G-1 decide, up to
+// four more draw the random numbers (Philox) into a ring per group, 16 LPC sites per
+// hand-off (one named barrier per group).
+//
+// Tests are made on integers, not predicates: the table holds thresholds and the lanes
+// hold draws shifted right by one, so that the sign of draw - threshold is the test, and
+// signs are combined with logic instructions (5 cycles a step, a predicate takes 13).  A
+// difference of zero leaves the test open (once in 2^31): the 32-bit table decides it.
 #pragma once
 #include "muca_internal.cuh"
 
@@ -46,8 +51,8 @@ static_assert(kMaxGroups < kFlushBarrier, "named barrier ids");
 __host__ __device__ constexpr int draw_warps(int groups) { return groups < 4 ? groups : 4; }
 __host__ __device__ constexpr int block_threads(int groups) { return 32 * (groups + draw_warps(groups)); }
 
-// Threshold table: in global memory, in shared memory, or in shared memory as the upper
-// 16 bits of each entry (a draw whose upper half ties its entry reads the 32-bit one).
+// Threshold table (31-bit entries): in global memory, in shared memory, or in shared memory
+// as the upper 16 bits of each threshold.
 enum Table { kTabGlobal = 0, kTabShared = 1, kTabShared16 = 2 };
 // Block histogram: in global memory, one 32-bit count per attempt, one per pair of
 // consecutive attempts (C[b][d + D]: the first ends in bin b, the second in b + d; D the
@@ -95,6 +100,17 @@ __device__ __forceinline__ uint32_t table_load(const char *ktab, uint32_t ad)
     }
     return v;
 }
+
+// 0xFF in byte i where the i-th argument is negative
+__device__ __forceinline__ uint32_t sign_bytes(uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    uint32_t x, y;
+    asm("prmt.b32 %0, %1, %2, 0x00FB;" : "=r"(x) : "r"(a), "r"(b));
+    asm("prmt.b32 %0, %1, %2, 0xFB00;" : "=r"(y) : "r"(c), "r"(d));
+    return __byte_perm(x, y, 0x7610);
+}
+// bits of t where m, of f elsewhere
+__device__ __forceinline__ uint32_t select(uint32_t m, uint32_t t, uint32_t f) { return (m & t) | (~m & f); }
 
 // bits 0..3 of x to bit 0 of the four bytes, and back
 __device__ __forceinline__ uint32_t spread4(uint32_t x) { return ((x & 0xFu) * 0x00204081u) & 0x01010101u; }
@@ -197,7 +213,7 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
     const int c0 = cblk * lw, n_own = max(0, min(lw, a.p - c0));  // first chain, chains of the block
 
     if (TAB == kTabShared)
-        for (int i = tid; i < n_tab; i += nt) s_tab[i] = a.ktab[i];
+        for (int i = tid; i < n_tab; i += nt) s_tab[i] = a.ktab[i] >> 1;
     if (TAB == kTabShared16)
         for (int i = tid; i < n_tab; i += nt) reinterpret_cast<uint16_t *>(s_tab)[i] = (uint16_t)(a.ktab[i] >> 16);
     for (int i = tid; i < n_hist; i += nt) s_hist[i] = 0u;
@@ -285,7 +301,7 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
         const uint32_t rowb = 4u * (uint32_t)a.row_words;  // bytes per lattice row
         const int nl = (L + 3) >> 2, jb = AL ? 3 : (L - 1) & 3;  // lanes' worth of sites per row, last site's byte
         const int nq = ROW ? 1 : (nl + LPC - 1) / LPC;     // passes per row
-        const char *const tab_g = reinterpret_cast<const char *>(a.ktab);
+        const char *const tab_g = reinterpret_cast<const char *>(a.ktab31);
         const uint32_t tab0 = TAB == kTabGlobal ? 0u : (uint32_t)__cvta_generic_to_shared(s_tab);
         const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring_of(grp));
         const uint32_t offs_s = (uint32_t)__cvta_generic_to_shared(offs_of(grp));
@@ -293,6 +309,7 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
         const uint32_t dummy = hist_s + 4u * (uint32_t)(((n_hist + 3) & ~3) + lane);
         const uint32_t starts = LPC == 4 ? 0x11111111u : LPC == 8 ? 0x01010101u : LPC == 16 ? 0x00010001u : 1u;
         const uint32_t prevbit = cl == 0 ? 0u : 1u << (lane - 1);
+        const int prevshift = (32 - lane) & 31;  // ... to bit 31
         // sums over the lanes of a chain: each lane's as a byte in shared memory, read back as
         // words and summed up to the lane by byte products (a shuffle scan takes twice as long)
         const uint32_t sums_s = (uint32_t)__cvta_generic_to_shared(s_ring) +
@@ -318,8 +335,12 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
             return POTTS ? raw & (vb * 255u) : spread4(raw >> (4 * (qi & 1))) & vb;
         };
 
-        int y = 0, q = 0, qi = cl;  // row, pass of the row, quad of the row
-        uint32_t vb = valid_of(qi);
+        int y = 0, q = 0, qi = cl;  // (long rows) row, pass of the row; quad of the row
+        uint32_t vb = valid_of(qi), vm = vb * 255u;
+        // (ROW) this lane's spins of the rows being decided and three rows on: byte offsets
+        uint8_t *const own = lat + (POTTS ? 4 * min(cl, nl - 1) : min(cl, nl - 1) >> 1);
+        const uint32_t allb = rowb * (uint32_t)L;
+        uint32_t o0 = 0u, o3 = L > 3 ? 3u * rowb : 0u;
         // neighbouring quads: shuffle sources and byte selectors (a row's ends wrap)
         const int base = ch * LPC;
         const int rsrc = ROW ? base + (cl >= nl - 1 ? 0 : cl + 1) : lane + 1;
@@ -331,7 +352,8 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
         const uint32_t wjb = COLB << (8 * jb);
         const uint32_t basebit = 1u << base;
 
-        uint32_t u[4], offn = 0u;
+        constexpr int SH = TAB == kTabShared16 ? 16 : 1;
+        uint32_t u[4], offn = 0u;  // draws >> SH, as the table's entries
         auto load_draws = [&](int pos) {
             const uint32_t s = ring_s + 4u * (uint32_t)(pos + 4 * cl);
             if (AL || (pos & 3) == 0) {
@@ -342,6 +364,8 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
 #pragma unroll
                 for (int i = 0; i < 4; ++i) u[i] = lds32(s + 4u * i);
             }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) u[i] >>= SH;
         };
         auto load_offsets = [&](int pos) {
             const uint32_t o = offs_s + (uint32_t)((pos & ~3) + 4 * cl);
@@ -401,7 +425,9 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
         auto upper = [&](uint32_t U, uint32_t X, uint32_t S) { return POTTS ? zs(U, X, S) : U ^ X; };
 
         // ---- the first pass
-        int pos = 0, lin = ROW ? L : min(4 * LPC, L), next_sync = Rg::kPhase, sw = 0;
+        int pos = 0, sw = 0;
+        // draws handed off and not yet in a pass; hand-offs taken
+        int ahead = Rg::kPhase - (ROW ? L : min(4 * LPC, L)), taken = 1;
         bar_sync(1 + grp, 64);
         load_draws(0);
         if (POTTS) load_offsets(0);
@@ -439,20 +465,22 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
             const bool lastq = ROW || q == nq - 1;
             // ---- the next pass: what does not depend on this one's decisions
             int y1 = y, q1 = q + 1;
-            if (lastq) {
+            if (!ROW && lastq) {
                 q1 = 0;
                 y1 = y + 1 == L ? 0 : y + 1;
             }
+            const bool last_row = ROW ? o0 + rowb == allb : y == L - 1;
             const int qi1 = ROW ? cl : q1 * LPC + cl;
             // its draws
             const int len = ROW ? L : min(4 * LPC, L - 4 * LPC * q), len1 = ROW ? L : min(4 * LPC, L - 4 * LPC * q1);
-            const int skip = !AL && lastq && y1 == 0 ? VS - V : 0;
+            const int skip = !AL && lastq && last_row ? VS - V : 0;
             int pos1 = pos + len + skip;
             pos1 = pos1 >= Rg::kSites ? pos1 - Rg::kSites : pos1;
-            lin += skip + len1;
-            if (lin > next_sync) {
-                if (next_sync < phases * Rg::kPhase) bar_sync(1 + grp, 64);
-                next_sync += Rg::kPhase;
+            ahead -= skip + len1;
+            if (ahead < 0) {
+                if (taken < phases) bar_sync(1 + grp, 64);
+                ++taken;
+                ahead += Rg::kPhase;
             }
             if (POTTS) load_offsets(pos1);
             uint32_t D1 = 0u, vb1 = vb, rsel1 = rselw, lsel1 = lselw, U1 = 0u, rr = 0u, ll = 0u;
@@ -469,54 +497,50 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
             }
 
             // ---- predict
-            bool flip = false;  // (ROW) site 0 is changed, and this lane has the row's last site
+            // (ROW) all ones in the lane of the row's last site if site 0 is changed: site 0's
+            // test is exact (its bin is the pass's first; an open one is found below), and the
+            // last site's right neighbour is fixed by it
+            uint32_t flip = 0u;
             if (ROW) {
-                // site 0's test is exact (its bin is the pass's first); it fixes the right
-                // neighbour of the row's last site
-                // (but for ties of 16-bit entries: the verification finds and corrects those)
-                const bool t0 = (TAB == kTabShared16 ? u[0] >> 16 : u[0]) < A0[0];
-                flip = (__ballot_sync(~0u, t0) & basebit) != 0u && lastm;
-                n0 += flip ? dalt : 0u;
-                n1 += flip ? dalt : 0u;
+                const bool f = (__ballot_sync(~0u, (int)(u[0] - A0[0]) < 0) & basebit) != 0u && lastm;
+                flip = f ? ~0u : 0u;
+                n0 += dalt & flip;
+                n1 += dalt & flip;
                 if (!AL) {
 #pragma unroll
                     for (int i = 0; i < 3; ++i) {
-                        A0[i] = flip && i == jb ? B0 : A0[i];
-                        A1[i] = flip && i == jb ? B1 : A1[i];
+                        A0[i] = f && i == jb ? B0 : A0[i];
+                        A1[i] = f && i == jb ? B1 : A1[i];
                     }
                 }
             }
-            uint32_t db, Rw, Q, e, k0, k1, da, SNr = 0u, SNl = 0u;
+            uint32_t dm, Rw, Q, e, k0, k1, da, SNr = 0u, SNl = 0u, nib = 0u;
             int bin1, binw;
             for (;;) {
-                // the lane's four sites for either incoming bit, then the incoming bits
-                uint32_t d0 = 0u, d1 = 0u, b0, b1;
+                // the lane's four sites for either incoming bit (signs: 0 kept, 1 changed), then
+                // the incoming bits
+                uint32_t d0, d1, b0, b1;
                 {
-                    bool s0 = false, s1 = true;
+                    uint32_t f0[4], f1[4];
+                    f0[0] = u[0] - A0[0];
+                    f1[0] = u[0] - A1[0];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const uint32_t x = TAB == kTabShared16 ? u[i] >> 16 : u[i];
-                        const bool p = x < A0[i], r = x < A1[i];
-                        bool f0 = s0 ? r : p, f1 = s1 ? r : p;
-                        if (ROW && AL && i == 3) {
-                            // (the last lane's outgoing bits are not used, so that only its own
-                            // last decision waits for site 0's)
-                            const bool pb = x < B0, rb = x < B1;
-                            const bool g0 = s0 ? rb : pb, g1 = s1 ? rb : pb;
-                            b0 = __ballot_sync(~0u, f0);
-                            b1 = __ballot_sync(~0u, f1);
-                            f0 = flip ? g0 : f0;
-                            f1 = flip ? g1 : f1;
-                        }
-                        if (f0) d0 |= 1u << (8 * i);
-                        if (f1) d1 |= 1u << (8 * i);
-                        s0 = f0;
-                        s1 = f1;
+                    for (int i = 1; i < 4; ++i) {
+                        const uint32_t p = u[i] - A0[i], r = u[i] - A1[i];
+                        f0[i] = select(f0[i - 1], r, p);
+                        f1[i] = select(f1[i - 1], r, p);
                     }
-                    if (!(ROW && AL)) {
-                        b0 = __ballot_sync(~0u, s0);
-                        b1 = __ballot_sync(~0u, s1);
+                    b0 = __ballot_sync(~0u, (int)f0[3] < 0);
+                    b1 = __ballot_sync(~0u, (int)f1[3] < 0);
+                    if (ROW && AL) {
+                        // (the last lane's outgoing bits are not used, so that only its own last
+                        // decision waits for site 0's)
+                        const uint32_t p = u[3] - B0, r = u[3] - B1;
+                        f0[3] = select(flip, select(f0[2], r, p), f0[3]);
+                        f1[3] = select(flip, select(f1[2], r, p), f1[3]);
                     }
+                    d0 = sign_bytes(f0[0], f0[1], f0[2], f0[3]);
+                    d1 = sign_bytes(f1[0], f1[1], f1[2], f1[3]);
                 }
                 // (the next pass's spins, neighbours and columns fill the gaps of this chain)
                 uint32_t RN1, LP1;
@@ -544,12 +568,12 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                     b0 = x;
                     b1 = z;
                 }
-                const bool cin = (b0 & prevbit) != 0u;
-                db = (cin ? d1 : d0) & vb;
+                // (all ones where the lane before ends with a change)
+                const uint32_t cin = (uint32_t)((int)((b0 & prevbit) << prevshift) >> 31);
+                dm = select(cin, d1, d0) & vm;
                 // columns of the sites as they were met, bin changes plus EB
-                const uint32_t lm = (db * 256u + (cin ? 1u : 0u)) * 255u;
-                const uint32_t N = (n1 & lm) | (n0 & ~lm), dm = db * 255u;
-                e = POTTS ? (N & dm) | (EB * m & ~dm) : ((4u * m - N) & dm) | (EB * m & ~dm);
+                const uint32_t lm = __byte_perm(dm, cin, 0x2104), N = select(lm, n1, n0);
+                e = select(dm, POTTS ? N : 4u * m - N, EB * m);
                 // sums over the lane's sites and the chain's lanes: bins before (X) and after (Q)
                 // every attempt are binw + byte
                 const uint32_t s = e * m;
@@ -587,41 +611,45 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                     uint32_t ad = __dp4a(N, COLB << (8 * i), __dp4a(X, ROWB << (8 * i), rw));
                     T[i] = table_load<TAB>(tab_g, ad);
                 }
-                Rw = POTTS ? (R & ~dm) | (SN & dm) : R ^ db;
+                Rw = POTTS ? select(dm, SN, R) : R ^ (dm & m);
+                if (!POTTS) {
+                    nib = pack4(Rw);
+                    nib |= __shfl_down_sync(~0u, nib, 1) << 4;
+                }
                 if (!ROW) {
                     // the row's first quad, and the quad before the next pass
                     const uint32_t fw = __shfl_sync(~0u, Rw, 0), pv = __shfl_sync(~0u, Rw, 31);
                     columns(R1, SN1, D1, qi1 == nl - 1 ? (q == 0 ? fw : first) : RN1, lane == 0 && q1 > 0 ? pv : LP1, 0u,
                             SNl, rsel1, lsel1, k0, k1, da);
                 }
-                uint32_t acc = 0u;
-                bool tie = false;
+                uint32_t df[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const uint32_t x = TAB == kTabShared16 ? u[i] >> 16 : u[i];
-                    if (x < T[i]) acc |= 1u << (8 * i);
-                    if (TAB == kTabShared16) tie |= x == T[i];
-                }
-                bool bad = ((acc ^ db) & vb) != 0u;
-                if (!__any_sync(~0u, bad || (TAB == kTabShared16 && tie && vb))) break;
-                if (TAB == kTabShared16) {
-                    // upper halves equal to their entries': the 32-bit tests decide
-                    acc = 0u;
+                for (int i = 0; i < 4; ++i) df[i] = u[i] - T[i];
+                const uint32_t open = min(min(df[0], df[1]), min(df[2], df[3]));  // zero: a test is open
+                uint32_t bad = (sign_bytes(df[0], df[1], df[2], df[3]) ^ dm) & vm;
+                if (!__any_sync(~0u, bad != 0u || open == 0u)) break;
+                if (__any_sync(~0u, open == 0u)) {
+                    // draws that equal their entries: the 32-bit tests decide
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
-                        const uint32_t b = (uint32_t)binw + ((X >> (8 * i)) & 0xFFu);
-                        const uint32_t A = vb & (1u << (8 * i)) ? __ldg(a.ktab + NC * b + ((N >> (8 * i)) & 0xFFu)) : 0u;
-                        if (u[i] < A) acc |= 1u << (8 * i);
-                        T[i] = u[i] < A ? 0x10000u : 0u;  // (what a repair compares 16 bits with)
+                        if (df[i] == 0u && vb & (1u << (8 * i))) {
+                            const uint32_t b = (uint32_t)binw + ((X >> (8 * i)) & 0xFFu);
+                            const uint32_t A = __ldg(a.ktab + NC * b + ((N >> (8 * i)) & 0xFFu));
+                            T[i] = lds32(ring_s + 4u * (uint32_t)(pos + 4 * cl + i)) < A ? 0x80000000u : 0u;
+                            df[i] = u[i] - T[i];
+                        }
                     }
-                    bad = ((acc ^ db) & vb) != 0u;
-                    // site 0 (its neighbours and bin are exact): what the last site saw of it
-                    const bool flip1 = (__ballot_sync(~0u, acc & 1u) & basebit) != 0u && lastm;
-                    n0 += flip1 == flip ? 0u : flip1 ? dalt : 0u - dalt;
-                    n1 += flip1 == flip ? 0u : flip1 ? dalt : 0u - dalt;
-                    bad = bad || flip1 != flip;
-                    flip = flip1;
-                    if (!__any_sync(~0u, bad)) break;
+                    bad = (sign_bytes(df[0], df[1], df[2], df[3]) ^ dm) & vm;
+                    if (ROW) {
+                        // site 0 (its neighbours and bin are exact): what the last site saw of it
+                        const bool f = (__ballot_sync(~0u, (int)df[0] < 0) & basebit) != 0u && lastm;
+                        const uint32_t flip1 = f ? ~0u : 0u;
+                        n0 += (dalt & flip1) - (dalt & flip);
+                        n1 += (dalt & flip1) - (dalt & flip);
+                        bad |= flip1 ^ flip;
+                        flip = flip1;
+                    }
+                    if (!__any_sync(~0u, bad != 0u)) break;
                 }
                 // repair: the verified thresholds, for the left neighbours as met
 #pragma unroll
@@ -647,12 +675,11 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
             }
             // ---- commit
             {
-                uint8_t *const r = lat + (size_t)y * rowb;
+                uint8_t *const r = ROW ? own + o0 : lat + (size_t)y * rowb + (POTTS ? 4 * qi : qi >> 1);
                 if (POTTS) {
-                    if (vb) *reinterpret_cast<volatile uint32_t *>(r + 4 * qi) = Rw;
+                    if (vb) *reinterpret_cast<volatile uint32_t *>(r) = Rw;
                 } else {
-                    const uint32_t nib = pack4(Rw), hi = __shfl_down_sync(~0u, nib, 1);
-                    if (vb && !(cl & 1)) *reinterpret_cast<volatile uint8_t *>(r + (qi >> 1)) = (uint8_t)(nib | (hi << 4));
+                    if (vb && !(cl & 1)) *reinterpret_cast<volatile uint8_t *>(r) = (uint8_t)nib;
                 }
             }
             __syncwarp();  // other lanes read these spins
@@ -709,7 +736,7 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                 }
             }
             if (lastq) {
-                if (record && y == L - 1) {
+                if (record && last_row) {
                     int M;
                     if (POTTS) {
                         counts.flush();
@@ -756,10 +783,16 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
             SN = SN1;
             if (ROW) {
                 R1 = D1;
-                const int y3 = y + 3;  // (now that row y is final: the row below the pass after next)
-                raw2 = raw_load(y3 >= L ? y3 - L : y3, cl);
+                // (now that this row is final: the row below the pass after next)
+                raw2 = POTTS ? *reinterpret_cast<const volatile uint32_t *>(own + o3)
+                             : (uint32_t) * reinterpret_cast<const volatile uint8_t *>(own + o3);
+                o0 = last_row ? 0u : o0 + rowb;
+                o3 = o3 + rowb == allb ? 0u : o3 + rowb;
             }
-            vb = vb1;
+            if (!ROW) {
+                vb = vb1;
+                vm = vb * 255u;
+            }
             qi = qi1;
             y = y1;
             q = q1;

@@ -274,6 +274,7 @@ int launch_sweeps(muca_ctx *ctx, uint32_t phase, int n_sweeps, uint32_t sweep0, 
     a.cnt = ctx->d_cnt;
     a.thr = ctx->d_thr;
     a.ktab = ctx->d_ktab;
+    a.ktab31 = ctx->d_ktab + (size_t)ctx->n_bins * ktab_width(ctx->model);
     a.H = ctx->d_H;
     a.samples = samples ? ctx->d_samples : nullptr;
     a.L = ctx->L;

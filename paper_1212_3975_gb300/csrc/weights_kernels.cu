@@ -61,6 +61,7 @@ __global__ void ktab_kernel(const uint32_t *thr, uint32_t *ktab, int model, int 
         v = dE == 0 ? kAlways : thr[b * 8 + (dE < 0 ? dE + 4 : dE + 3)];
     }
     ktab[t] = v;
+    ktab[n_bins * width + t] = v >> 1;  // (as the sweep bodies compare them)
 }
 
 struct BlockStats {
