@@ -244,10 +244,11 @@ constexpr int kRwTile = 8;          // betas per tile
 constexpr int kRwMaxChunks = 32;    // bin chunks per tile at most
 constexpr size_t kRwTileParamsBytes = 72;
 constexpr size_t rw_align256(size_t b) { return (b + 255) & ~(size_t)255; }
-// per-bin part: five FP64 arrays, five float arrays (ln Omega and mean |M| as float
-// pairs, the within-bin variance), the sampled range of every block of the preparation
-// kernel (256 bins each), and the completion counter of the setup kernel (zero between
-// calls: zeroed with the scratch, reset by its last user)
+// per-bin part: five FP64 arrays (the second, bin energies, is the BF16 path's; the tiled
+// kernels keep the sampled range of every 64 bins there), five float arrays (ln Omega and
+// mean |M| as float pairs, the within-bin variance), a free piece of 8 bytes per 256 bins
+// (callers know the size of the whole), and the completion counter of the setup kernel
+// (zero between calls: zeroed with the scratch, reset by its last user)
 constexpr size_t rw_bin_part_bytes(size_t nb)
 {
     return rw_align256(5 * nb * 8) + 5 * rw_align256(nb * 4) + rw_align256(8 * ((nb + 255) / 256)) + 256;

@@ -18,15 +18,17 @@
 //      the tile, and a per-beta shift c_t (the negated maximum of the exponent).
 //      Any shift common to all bins of a beta cancels in <X> = sum w X / sum w, so an
 //      approximate (FP32) maximum is enough: it only keeps the exponents in range.
-//   3. scan: the tiles' bin windows are cut into chunks (at most 32 per tile) and
-//      numbered, so that
+//   3. scan: the tiles' bin windows are cut into chunks (some six items per SM in all,
+//      at most 32 per tile) and numbered, so that
 //   4. sums: a persistent grid fills every SM with (tile, chunk) items, each writing
 //      FP64 partial sums of the six centred columns for the tile's betas;
 //   5. combine: per beta, the partial sums in chunk order (deterministic), then the
 //      observables.
 // The exponent of bin b at beta_t is a = G_b + c_t - (beta_t - beta_T)(E_b - E_kT) with
 // G_b = lnOmega_b - lnOmega_kT - beta_T (E_b - E_kT) formed in FP64 once per (tile,
-// bin).  MUCA_FP64 evaluates a and exp(a) in FP64 and skips a < -100.  MUCA_FP32
+// bin).  MUCA_FP64 takes exp(a) as exp(G_b) times powers of exp(beta_T - beta_t), or,
+// where a tile's betas lie too far apart for that, evaluates a and exp(a) per term and
+// skips a < -100.  MUCA_FP32
 // evaluates a as an unevaluated sum of two floats (G_b and beta_t - beta_T split into
 // high and low floats, the product by the exact integer E_b - E_kT with its FMA-exact
 // error, error-free additions) and w = exp2(a_hi) (1 + a_lo ln 2): at a beta far from
@@ -333,7 +335,8 @@ struct RwScratch {
     float *lnOl;                   //   and low part of lnOmega as a float pair
     float *x1h, *x1l;              // mean |M| as a float pair
     float *vf;                     // within-bin variance of |M| (float)
-    int2 *blkrange;                // [ceil(n_bins / 256)] lowest / highest sampled bin of each prep block
+    int2 *blkrange;                // [nblk] lowest / highest sampled bin of each prep block (in the
+                                   //   array of the bin energies, which the tiled kernels do not read)
     int nblk;
     TileParams *tiles;             // [n_tiles]
     double *c;                     // [n_beta] per-beta shift (ln units)
@@ -345,29 +348,40 @@ struct RwScratch {
     unsigned *cnt0;                // completion counter of the setup kernel (zero between calls)
     unsigned *cnt;                 // [n_tiles] completion counters of the tiles (zeroed by the setup)
     int *item_tile;                // [n_tiles * kRwMaxChunks] tile of every item
-    double *part;                  // [n_tiles * kRwMaxChunks][kRwTile][6] partial sums
+    double *part;                  // [n_tiles * kRwChunks][kRwTile][6] partial sums
+    double *pow;                   // [n_tiles][kRwPow] powers of the tiles' betas (in part's last slots)
 };
+
+// Of a tile's kRwMaxChunks slots of partial sums the last six hold its powers (FP64):
+// exp(-(beta_t - beta_T) E) for the energies of 0..31 bins ([t][32]) and whether they
+// apply (1 or 0).
+constexpr int kRwChunks = kRwMaxChunks - 6;
+constexpr int kRwPow = 6 * kRwTile * 6;
+static_assert(kRwPow >= 32 * kRwTile + 1, "powers of a tile");
+constexpr int kPrepThreads = 64;    // bins per block of the preparation
 
 __device__ __forceinline__ double bin_energy(int model, int V, int b)
 {
     return model == MUCA_ISING ? (double)(4 * b - 2 * V) : (double)(b - 2 * V);
 }
 
-// Per bin: FP64 lnOmega and means, the float copy, and the block's sampled range.
-__global__ void __launch_bounds__(256) rw_prep_kernel(const uint64_t *samples, const double *lnw, RwScratch r,
-                                                      int model, int V, int n_bins)
+// Per bin: FP64 lnOmega and means, the float copy, and the block's sampled range.  A
+// bin's logarithm and two divisions are some hundred FP64 operations at two per clock
+// and SM, so the bins are dealt to as many SMs as there are (64 per block; 4097 bins:
+// 6.5 us, in blocks of 256 8.0 us).
+__global__ void __launch_bounds__(kPrepThreads) rw_prep_kernel(const uint64_t *samples, const double *lnw, RwScratch r,
+                                                               int n_bins)
 {
-    __shared__ int s_lo[8], s_hi[8];
+    __shared__ int2 s_range;
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     int lo = 0x7FFFFFFF, hi = -1;
     if (b < n_bins) {
         const uint64_t n = samples[b];
-        r.d.E[b] = bin_energy(model, V, b);
         if (n == 0) {
             r.d.lnO[b] = -INFINITY;
             r.lnOf[b] = -INFINITY;
             r.lnOl[b] = r.x1h[b] = r.x1l[b] = r.vf[b] = 0.f;
-            r.d.x1[b] = r.d.x2[b] = r.d.v[b] = 0.0;
+            r.d.x1[b] = r.d.v[b] = 0.0;
         } else {
             const double nd = (double)n;
             const double l = __dsub_rn(log(nd), lnw[b]);
@@ -378,7 +392,6 @@ __global__ void __launch_bounds__(256) rw_prep_kernel(const uint64_t *samples, c
             const double x1 = __ddiv_rn((double)samples[n_bins + b], nd);
             const double x2 = __ddiv_rn((double)samples[2 * n_bins + b], nd);
             r.d.x1[b] = x1;
-            r.d.x2[b] = x2;
             r.d.v[b] = x2 - x1 * x1;
             const float xh = (float)x1;
             r.x1h[b] = xh;
@@ -387,17 +400,11 @@ __global__ void __launch_bounds__(256) rw_prep_kernel(const uint64_t *samples, c
             lo = hi = b;
         }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-        hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) { s_lo[warp] = lo; s_hi[warp] = hi; }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (threadIdx.x == 32) s_range = make_int2(lo, hi);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < 8; ++w) { lo = min(lo, s_lo[w]); hi = max(hi, s_hi[w]); }
-        r.blkrange[blockIdx.x] = make_int2(lo, hi);
-    }
+    if (threadIdx.x == 0) r.blkrange[blockIdx.x] = make_int2(min(lo, s_range.x), max(hi, s_range.y));
 }
 
 __device__ __forceinline__ void warp_argmax(float &v, int &i)
@@ -409,11 +416,13 @@ __device__ __forceinline__ void warp_argmax(float &v, int &i)
     }
 }
 
-// Exclusive prefix of the tiles' chunk counts, by one block of 256 threads (the last
+// Exclusive prefix of the tiles' chunk counts, by one block of THREADS (the last
 // setup block); tiles without a sampled bin get NaN observables here.
+template <int THREADS>
 __device__ void scan_tiles(RwScratch &r, int n_tiles, int n_beta, Observables o)
 {
-    __shared__ int s_part[8];
+    constexpr int NW = THREADS / 32;
+    __shared__ int s_part[NW];
     __shared__ int s_carry;
     if (threadIdx.x == 0) s_carry = 0;
     __syncthreads();
@@ -432,12 +441,12 @@ __device__ void scan_tiles(RwScratch &r, int n_tiles, int n_beta, Observables o)
         if (lane == 31) s_part[warp] = x;
         __syncthreads();
         if (warp == 0) {
-            int w = lane < 8 ? s_part[lane] : 0;
-            for (int k = 1; k < 8; k <<= 1) {
+            int w = lane < NW ? s_part[lane] : 0;
+            for (int k = 1; k < NW; k <<= 1) {
                 const int y = __shfl_up_sync(0xffffffffu, w, k);
                 if (lane >= k) w += y;
             }
-            if (lane < 8) s_part[lane] = w;
+            if (lane < NW) s_part[lane] = w;
         }
         __syncthreads();
         const int incl = x + (warp > 0 ? s_part[warp - 1] : 0) + s_carry;
@@ -452,64 +461,65 @@ __device__ void scan_tiles(RwScratch &r, int n_tiles, int n_beta, Observables o)
     if (threadIdx.x == 0) r.off[n_tiles] = s_carry;
 }
 
-// One block (256 threads) per tile: reference bin, window, chunks and per-beta shifts,
-// in two passes over the sampled bins; the block that finishes last numbers the chunks
-// of all tiles.
-__global__ void __launch_bounds__(256) rw_setup_kernel(RwScratch r, const double *betas, int n_beta, int model, int V,
-                                                       Observables o)
+// One block per tile: reference bin, window, chunks and per-beta shifts, in two passes
+// over the sampled bins; the block that finishes last numbers the chunks of all tiles.
+// Bound by the latency of the passes' loads and of the reductions: 512 threads take the
+// 4097 bins of a 64x64 lattice in eight loads each.  Two such blocks fit an SM (four of
+// 256 threads), so from more than two tiles per SM on, a tile has 256 (512 tiles: 15 us
+// against 20 with 512 threads; 64 tiles: 11 us against 18 with 256).
+// max_chunks: chunks per tile at most; powers: the sums are FP64.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS) rw_setup_kernel(RwScratch r, const double *betas,
+                                                                           int n_beta, int model, int V,
+                                                                           int max_chunks, bool powers, Observables o)
 {
-    __shared__ float s_v[8], s_m[8][kRwTile];
-    __shared__ int s_i[8], s_lo[8], s_hi[8], s_mi[8][kRwTile];
-    __shared__ int s_last;
+    constexpr int NW = THREADS / 32;
+    __shared__ float s_v[NW], s_m[NW][kRwTile], s_db[kRwTile];
+    __shared__ int s_i[NW], s_lo[NW], s_hi[NW], s_mi[NW][kRwTile];
+    __shared__ bool s_last;
     const int T = blockIdx.x, j0 = T * kRwTile, nt = min(kRwTile, n_beta - j0);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int dstep = model == MUCA_ISING ? 4 : 1;  // energy step between neighbouring bins
     if (threadIdx.x == 0) r.cnt[T] = 0u;  // the sums kernel counts this tile's chunks from zero
+    const double betaT = betas[j0 + nt / 2];
+    const float bTf = (float)betaT;
+    if ((int)threadIdx.x < kRwTile) s_db[threadIdx.x] = (int)threadIdx.x < nt ? (float)(betas[j0 + threadIdx.x] - betaT) : 0.f;
     // sampled range of the bins, from the preparation blocks' ranges
     int lo_s = 0x7FFFFFFF, hi_s = -1;
-    for (int i = threadIdx.x; i < r.nblk; i += blockDim.x) {
+    for (int i = threadIdx.x; i < r.nblk; i += THREADS) {
         const int2 br = r.blkrange[i];
         lo_s = min(lo_s, br.x);
         hi_s = max(hi_s, br.y);
     }
-    for (int k = 16; k > 0; k >>= 1) {
-        lo_s = min(lo_s, __shfl_xor_sync(0xffffffffu, lo_s, k));
-        hi_s = max(hi_s, __shfl_xor_sync(0xffffffffu, hi_s, k));
-    }
+    lo_s = __reduce_min_sync(0xffffffffu, lo_s);
+    hi_s = __reduce_max_sync(0xffffffffu, hi_s);
     if (lane == 0) { s_lo[warp] = lo_s; s_hi[warp] = hi_s; }
     __syncthreads();
-    lo_s = s_lo[0];
-    hi_s = s_hi[0];
-    for (int w = 1; w < 8; ++w) { lo_s = min(lo_s, s_lo[w]); hi_s = max(hi_s, s_hi[w]); }
-    __syncthreads();
-    const double betaT = betas[j0 + nt / 2];
-    const float bTf = (float)betaT;
+    lo_s = __reduce_min_sync(0xffffffffu, s_lo[lane % NW]);
+    hi_s = __reduce_max_sync(0xffffffffu, s_hi[lane % NW]);
+    if (hi_s < 0) lo_s = 0;  // no sampled bin at all
     // pass 1: approximate reference bin (FP32)
     float best = -INFINITY;
     int kT = max(0, hi_s);  // replaced by a sampled bin whenever there is one
-#pragma unroll 4
-    for (int b = lo_s + (int)threadIdx.x; b <= hi_s; b += 256) {
+    const int E0 = -2 * V;
+#pragma unroll 8
+    for (int b = lo_s + (int)threadIdx.x; b <= hi_s; b += THREADS) {
         const float l = r.lnOf[b];
-        const float a = l - bTf * (float)bin_energy(model, V, b);
+        const float a = l - bTf * (float)(E0 + dstep * b);
         if (l != -INFINITY && a > best) { best = a; kT = b; }
     }
     warp_argmax(best, kT);
     if (lane == 0) { s_v[warp] = best; s_i[warp] = kT; }
     __syncthreads();
-    if (threadIdx.x < 32) {
-        best = lane < 8 ? s_v[lane] : -INFINITY;
-        kT = lane < 8 ? s_i[lane] : max(0, hi_s);
-        warp_argmax(best, kT);
-        if (lane == 0) s_i[0] = kT;
-    }
-    __syncthreads();
-    kT = s_i[0];
+    best = s_v[lane % NW];
+    kT = s_i[lane % NW];
+    warp_argmax(best, kT);
     const float lTf = r.lnOf[kT];
     const double ETd = bin_energy(model, V, kT);
-    const float ETf = (float)ETd;
     float db[kRwTile], dbmax = 0.f;
 #pragma unroll
     for (int t = 0; t < kRwTile; ++t) {
-        db[t] = t < nt ? (float)(betas[j0 + t] - betaT) : 0.f;
+        db[t] = s_db[t];
         dbmax = fmaxf(dbmax, fabsf(db[t]));
     }
     // pass 2: the window (bins that can reach e^-100 of the largest weight for some beta
@@ -525,77 +535,85 @@ __global__ void __launch_bounds__(256) rw_setup_kernel(RwScratch r, const double
         mx[t] = -INFINITY;
         mi[t] = kT;
     }
-#pragma unroll 2
-    for (int b = lo_s + (int)threadIdx.x; b <= hi_s; b += 256) {
+#pragma unroll 4
+    for (int b = lo_s + (int)threadIdx.x; b <= hi_s; b += THREADS) {
         const float l = r.lnOf[b];
-        if (l == -INFINITY) continue;
-        const float dE = (float)bin_energy(model, V, b) - ETf;
-        const float G = (l - lTf) - bTf * dE;
-        if (G + dbmax * fabsf(dE) >= (float)kCut - 2.f) { lo = min(lo, b); hi = max(hi, b); }
+        if (l != -INFINITY) {
+            const float dE = (float)(dstep * (b - kT));
+            const float G = (l - lTf) - bTf * dE;
+            if (G + dbmax * fabsf(dE) >= (float)kCut - 2.f) { lo = min(lo, b); hi = max(hi, b); }
 #pragma unroll
-        for (int t = 0; t < kRwTile; ++t) {
-            const float v = G - db[t] * dE;
-            if (v > mx[t]) {
-                mx[t] = v;
-                mi[t] = b;
+            for (int t = 0; t < kRwTile; ++t) {
+                const float v = G - db[t] * dE;
+                if (v > mx[t]) {
+                    mx[t] = v;
+                    mi[t] = b;
+                }
             }
         }
     }
-    for (int k = 16; k > 0; k >>= 1) {
-        lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, k));
-        hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, k));
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    // the warp's maxima by halving (as in halving_sums): that of beta 4 (lane & 1) +
+    // 2 (lane >> 1 & 1) + (lane >> 2 & 1) ends in the lane
 #pragma unroll
-        for (int t = 0; t < kRwTile; ++t) {
-            const float ov = __shfl_xor_sync(0xffffffffu, mx[t], k);
-            const int oi = __shfl_xor_sync(0xffffffffu, mi[t], k);
-            if (ov > mx[t] || (ov == mx[t] && oi < mi[t])) {
-                mx[t] = ov;
-                mi[t] = oi;
+    for (int s = 0, n = kRwTile / 2; s < 5; ++s) {
+        const bool up = (lane >> s) & 1;
+#pragma unroll
+        for (int i = 0; i < kRwTile / 2; ++i) {
+            if (i < max(n, 1)) {
+                const bool swap = n > 0;
+                float kv = mx[i], ov = mx[i];
+                int ki = mi[i], oi = mi[i];
+                if (swap) {
+                    kv = up ? mx[i + n] : mx[i];
+                    ov = up ? mx[i] : mx[i + n];
+                    ki = up ? mi[i + n] : mi[i];
+                    oi = up ? mi[i] : mi[i + n];
+                }
+                ov = __shfl_xor_sync(0xffffffffu, ov, 1 << s);
+                oi = __shfl_xor_sync(0xffffffffu, oi, 1 << s);
+                const bool take = ov > kv || (ov == kv && oi < ki);
+                mx[i] = take ? ov : kv;
+                mi[i] = take ? oi : ki;
             }
         }
+        n >>= 1;
+    }
+    if (lane == 0) { s_lo[warp] = lo; s_hi[warp] = hi; }
+    if (lane < kRwTile) {
+        const int t = 4 * (lane & 1) + 2 * ((lane >> 1) & 1) + (lane >> 2);
+        s_m[warp][t] = mx[0];
+        s_mi[warp][t] = mi[0];
     }
     __syncthreads();
-    if (lane == 0) {
-        s_lo[warp] = lo;
-        s_hi[warp] = hi;
-#pragma unroll
-        for (int t = 0; t < kRwTile; ++t) {
-            s_m[warp][t] = mx[t];
-            s_mi[warp][t] = mi[t];
-        }
-    }
-    __syncthreads();
-    lo = s_lo[0];
-    hi = s_hi[0];
-    for (int w = 1; w < 8; ++w) { lo = min(lo, s_lo[w]); hi = max(hi, s_hi[w]); }
+    lo = __reduce_min_sync(0xffffffffu, s_lo[lane % NW]);
+    hi = __reduce_max_sync(0xffffffffu, s_hi[lane % NW]);
     if (lo > hi) {  // no sampled bin at all: an empty window
         lo = 0;
         hi = -1;
     }
-    if ((int)threadIdx.x < nt) {
-        const int t = threadIdx.x, j = j0 + t;
-        float m = s_m[0][t];
-        int k = s_mi[0][t];
-        for (int w = 1; w < 8; ++w)
-            if (s_m[w][t] > m || (s_m[w][t] == m && s_mi[w][t] < k)) {
-                m = s_m[w][t];
-                k = s_mi[w][t];
-            }
-        const double c = -(double)m;  // per-beta shift (ln units)
-        r.c[j] = c;
-        const double db2 = (betas[j] - betaT) * kLog2e;
-        const float dbh = (float)db2;
-        // the beta's reference: E_ref - E_T (an exact integer, also as a float) and the
-        // bin's mean |M|
-        const float dref = (float)(bin_energy(model, V, k) - ETd);
-        r.bc[j] = make_float4(dbh, (float)(db2 - (double)dbh), (float)(c * kLog2e), dref);
-        r.xref[j] = r.d.x1[k];
-        r.xrf[j] = make_float2(r.x1h[k], r.x1l[k]);
+    if (warp < nt) {
+        // a warp per beta
+        const int t = warp, j = j0 + t;
+        float m = s_m[lane % NW][t];
+        int k = s_mi[lane % NW][t];
+        warp_argmax(m, k);
+        if (lane == 0) {
+            const double c = -(double)m;  // per-beta shift (ln units)
+            r.c[j] = c;
+            const double db2 = (betas[j] - betaT) * kLog2e;
+            const float dbh = (float)db2;
+            // the beta's reference: E_ref - E_T (an exact integer, also as a float) and
+            // the bin's mean |M|
+            r.bc[j] = make_float4(dbh, (float)(db2 - (double)dbh), (float)(c * kLog2e), (float)(dstep * (k - kT)));
+            r.xref[j] = r.d.x1[k];
+            r.xrf[j] = make_float2(r.x1h[k], r.x1l[k]);
+        }
     }
-    if (threadIdx.x == 0) {
-        const int width = max(0, hi - lo + 1);
-        int ch = max(kRwMinChunk, (width + kRwMaxChunks - 1) / kRwMaxChunks);
-        ch = (ch + 31) & ~31;
+    const int width = max(0, hi - lo + 1);
+    const int ch = (max(kRwMinChunk, (width + max_chunks - 1) / max_chunks) + 31) & ~31;
+    if (threadIdx.x == THREADS - 32) {
         TileParams tp;
         tp.kT = kT;
         tp.lo = lo;
@@ -613,6 +631,16 @@ __global__ void __launch_bounds__(256) rw_setup_kernel(RwScratch r, const double
         tp.bTl = (float)(betaT - (double)tp.bTh);
         r.tiles[T] = tp;
     }
+    if (powers && warp >= NW - kRwTile) {
+        // they apply where every exponent stays far from the range of FP64, up to the
+        // end of the last chunk
+        const float reach = dbmax * (float)dstep * ((float)max(abs(lo - kT), abs(hi - kT)) + (float)ch);
+        double *pw = r.pow + (size_t)T * kRwPow;
+        const int t = warp - (NW - kRwTile);
+        const double step = t < nt ? (betas[j0 + t] - betaT) * (double)dstep : 0.0;
+        if (reach <= 300.f) pw[32 * t + lane] = exp(-step * (double)lane);
+        if (t == 0 && lane == 0) pw[32 * kRwTile] = reach <= 300.f ? 1.0 : 0.0;
+    }
     // the last block to finish numbers the chunks (the classic last-block pattern: no
     // block waits for another)
     __threadfence();
@@ -621,7 +649,7 @@ __global__ void __launch_bounds__(256) rw_setup_kernel(RwScratch r, const double
     __syncthreads();
     if (s_last) {
         __threadfence();
-        scan_tiles(r, gridDim.x, n_beta, o);
+        scan_tiles<THREADS>(r, gridDim.x, n_beta, o);
         if (threadIdx.x == 0) *r.cnt0 = 0u;
     }
 }
@@ -633,19 +661,62 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
 
-// Persistent grid over the (tile, chunk) items.  FP64: exponents, weights and sums in
-// FP64.  FP32: compensated exponents and weights in FP32; every column sum is kept as a
-// float pair (high part and the accumulated rounding errors of its additions), through
-// the thread's bins and the warp's tree, and combined in FP64 across warps.  (Plain
-// FP32 sums of 32 terms lost up to ~1e-6 relative on C and chi.)
-template <bool FP64>
-__global__ void __launch_bounds__(256) rw_sums_kernel(RwScratch r, const double *betas, int n_beta, int n_tiles,
-                                                      int model, int V, double mnorm, Observables o)
+// Sums over the 32 lanes of 24 values per lane by halving: a step sends one half of the
+// values and adds the other half received, so a lane makes 27 additions instead of 120
+// (the sums of an item's few bins per thread cost more than its terms otherwise; in FP64
+// an addition is 64 cycles of a scheduler).  Value 12 (lane & 1) + 6 (lane >> 1 & 1) +
+// 3 (lane >> 2 & 1) + i ends in v[i] of the lane, i = 0..2.
+template <typename V, typename Shuffle, typename Add>
+__device__ __forceinline__ void halving_sums(V (&v)[24], int lane, Shuffle shuffle, Add add)
 {
-    __shared__ double s_red[8][kRwTile][6];
-    __shared__ float2 s_rf[8][kRwTile][6];
+#pragma unroll
+    for (int s = 0, n = 12; s < 3; ++s, n >>= 1) {
+        const bool up = (lane >> s) & 1;
+#pragma unroll
+        for (int i = 0; i < 12; ++i) {
+            if (i < n) {
+                const V keep = up ? v[i + n] : v[i], send = up ? v[i] : v[i + n];
+                v[i] = add(keep, shuffle(send, 1 << s));
+            }
+        }
+    }
+#pragma unroll
+    for (int s = 8; s <= 16; s <<= 1)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) v[i] = add(v[i], shuffle(v[i], s));
+}
+__device__ __forceinline__ int halving_index(int lane)
+{
+    return 12 * (lane & 1) + 6 * ((lane >> 1) & 1) + 3 * ((lane >> 2) & 1);
+}
+
+// Persistent grid over the (tile, chunk) items.  Warps 0..3 take the tile's betas 0..3,
+// warps 4..7 betas 4..7 (sums of eight betas per thread need all 255 registers and spill:
+// one block per SM), four bins of a warp's 32 at a time.
+// FP64: the weight of bin b at beta_t is exp(G_b) (once per tile and bin) times a power
+// of the beta's offset, exp(c_t - (beta_t - beta_T) E): the product of a power for the
+// warp's first bin and one for the lane (the setup's table), two products per term
+// instead of an exponential (some twenty FP64 operations at two per clock and SM).
+// Tiles whose exponents reach too far take the exponential of every term.  FP32:
+// compensated exponents and weights in FP32; every column sum is kept as a float pair
+// (high part and the accumulated rounding errors of its additions), through the thread's
+// bins and the warp's sums, and combined in FP64 across warps.  (Plain FP32 sums of 32
+// terms lost up to ~1e-6 relative on C and chi.)
+// Bound by the FP64 pipe (two per clock and SM; ~12 per term, besides exponentials and
+// sums) and by instruction issue in FP32 (~70 per term).  512 betas on the 4097 bins of
+// 64x64, FP64: 84 us with an exponential per term, sums of 120 additions and chunks of
+// 128 bins, 33 us now; 4096 betas on the canonical window of 256x256, FP32: 173 -> 33 us.
+template <bool FP64>
+__global__ void __launch_bounds__(256, 2) rw_sums_kernel(RwScratch r, const double *betas, int n_beta, int n_tiles,
+                                                         int model, int V, double mnorm, Observables o)
+{
+    constexpr int TB = kRwTile / 2;
+    static_assert(TB * 6 == 24, "halving_sums");
+    __shared__ double s_red[FP64 ? 8 : 1][TB * 6];
+    __shared__ double s_g[2][FP64 ? 256 : 1], s_ph[2][2][FP64 ? 32 : 1];
+    __shared__ float2 s_rf[FP64 ? 1 : 8][TB * 6];
     __shared__ int s_done;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t0 = TB * (warp >> 2);
     const int total = r.off[n_tiles];
     const int dstep = model == MUCA_ISING ? 4 : 1;  // energy step between neighbouring bins
     const int n_bins = model == MUCA_ISING ? V + 1 : 2 * V + 1;
@@ -658,61 +729,100 @@ __global__ void __launch_bounds__(256) rw_sums_kernel(RwScratch r, const double 
         // chunks are whole multiples of 32 bins: the last one may reach past the last
         // bin, where the per-bin arrays end (the next array follows directly)
         const int b1 = min(min(b0 + tp.ch, tp.lo + tp.nch * tp.ch), n_bins);
+        const int bw = b0 + 32 * (warp & 3);  // the warp's first bin
         if (FP64) {
-            double cd[kRwTile], dbd[kRwTile], drd[kRwTile], xrd[kRwTile];
+            double cd[TB], dbd[TB], drd[TB], xrd[TB], acc[TB * 6];
 #pragma unroll
-            for (int t = 0; t < kRwTile; ++t) {
-                const bool ok = t < nt;
-                cd[t] = ok ? r.c[j0 + t] : -1e300;
-                dbd[t] = ok ? betas[j0 + t] - tp.betaT : 0.0;
-                drd[t] = ok ? (double)r.bc[j0 + t].w : 0.0;
-                xrd[t] = ok ? r.xref[j0 + t] : 0.0;
-            }
-            double acc[kRwTile][6];
-#pragma unroll
-            for (int t = 0; t < kRwTile; ++t)
-#pragma unroll
-                for (int k = 0; k < 6; ++k) acc[t][k] = 0.0;
-            for (int b = b0 + (int)threadIdx.x; b < b1; b += blockDim.x) {
-                const double l = r.d.lnO[b];
-                if (l == -INFINITY) continue;
-                const double dEd = (double)(dstep * (b - tp.kT));
-                const double G = __dsub_rn(__dsub_rn(l, tp.lnOT), __dmul_rn(tp.betaT, dEd));
-                const double x1 = r.d.x1[b], vb = r.d.v[b];
-#pragma unroll
-                for (int t = 0; t < kRwTile; ++t) {
-                    const double a = __fma_rn(-dbd[t], dEd, G + cd[t]);
-                    if (a < kCut) continue;
-                    const double w = exp(a);
-                    // columns centred on the beta's reference bin
-                    const double d = dEd - drd[t], dx = x1 - xrd[t];
-                    const double cols[6] = {1.0, d, d * d, dx, dx * dx, vb};
-#pragma unroll
-                    for (int k = 0; k < 6; ++k) acc[t][k] = __fma_rn(w, cols[k], acc[t][k]);
-                }
+            for (int t = 0; t < TB; ++t) {
+                const bool ok = t0 + t < nt;
+                const int j = j0 + t0 + t;
+                cd[t] = ok ? r.c[j] : -1e300;
+                dbd[t] = ok ? betas[j] - tp.betaT : 0.0;
+                drd[t] = ok ? (double)r.bc[j].w : 0.0;
+                xrd[t] = ok ? r.xref[j] : 0.0;
             }
 #pragma unroll
-            for (int t = 0; t < kRwTile; ++t)
+            for (int k = 0; k < TB * 6; ++k) acc[k] = 0.0;
+            auto add_term = [&](int t, double w, double dEd, double x1, double vb) {
+                // columns centred on the beta's reference bin
+                const double d = dEd - drd[t], dx = x1 - xrd[t];
+                acc[6 * t] += w;
+                acc[6 * t + 1] = __fma_rn(w, d, acc[6 * t + 1]);
+                acc[6 * t + 2] = __fma_rn(w, d * d, acc[6 * t + 2]);
+                acc[6 * t + 3] = __fma_rn(w, dx, acc[6 * t + 3]);
+                acc[6 * t + 4] = __fma_rn(w, dx * dx, acc[6 * t + 4]);
+                acc[6 * t + 5] = __fma_rn(w, vb, acc[6 * t + 5]);
+            };
+            const double *pw = r.pow + (size_t)T * kRwPow;
+            if (pw[32 * kRwTile] != 0.0) {
+                double pl[TB];
 #pragma unroll
-                for (int k = 0; k < 6; ++k) {
-                    double x = acc[t][k];
-                    for (int q = 16; q > 0; q >>= 1) x += __shfl_xor_sync(0xffffffffu, x, q);
-                    if (lane == 0) s_red[warp][t][k] = x;
+                for (int t = 0; t < TB; ++t) pl[t] = pw[32 * (t0 + t) + lane];
+                // 256 bins at a time: exp(G_b) one per thread, the powers of the first
+                // bins of every 32 by two warps, then two times 128 bins
+                int buf = 0;
+                for (int bb = b0; bb < b1; bb += 256, buf ^= 1) {
+                    const int b = bb + (int)threadIdx.x;
+                    const double l = b < b1 ? r.d.lnO[b] : -INFINITY;
+                    double g = 0.0;
+                    if (l != -INFINITY)
+                        g = exp(__dsub_rn(__dsub_rn(l, tp.lnOT), __dmul_rn(tp.betaT, (double)(dstep * (b - tp.kT)))));
+                    s_g[buf][threadIdx.x] = g;
+                    if (warp < 2) {
+                        const int t = lane >> 2, j = min(j0 + t, n_beta - 1);
+                        const double x = t < nt ? r.c[j] : -1e300, d = t < nt ? betas[j] - tp.betaT : 0.0;
+                        s_ph[buf][warp][lane] =
+                            exp(__fma_rn(-d, (double)(dstep * (bb + 128 * warp + 32 * (lane & 3) - tp.kT)), x));
+                    }
+                    __syncthreads();
+#pragma unroll
+                    for (int s = 0; s < 2; ++s) {
+                        const int i = 128 * s + 32 * (warp & 3) + lane;
+                        const double gs = s_g[buf][i];
+                        if (!__any_sync(~0u, gs != 0.0)) continue;
+                        const double dEd = (double)(dstep * (bb + i - tp.kT));
+                        const bool in = bb + i < b1;
+                        const double x1 = in ? r.d.x1[bb + i] : 0.0, vb = in ? r.d.v[bb + i] : 0.0;
+#pragma unroll
+                        for (int t = 0; t < TB; ++t)
+                            add_term(t, gs * (pl[t] * s_ph[buf][s][4 * (t0 + t) + (warp & 3)]), dEd, x1, vb);
+                    }
                 }
+            } else {
+                for (int b = bw + lane; b < b1; b += 128) {
+                    const double l = r.d.lnO[b];
+                    if (l == -INFINITY) continue;
+                    const double dEd = (double)(dstep * (b - tp.kT));
+                    const double G = __dsub_rn(__dsub_rn(l, tp.lnOT), __dmul_rn(tp.betaT, dEd));
+                    const double x1 = r.d.x1[b], vb = r.d.v[b];
+#pragma unroll
+                    for (int t = 0; t < TB; ++t) {
+                        const double a = __fma_rn(-dbd[t], dEd, G + cd[t]);
+                        if (a < kCut) continue;
+                        add_term(t, exp(a), dEd, x1, vb);
+                    }
+                }
+            }
+            halving_sums(acc, lane, [](double x, int s) { return __shfl_xor_sync(~0u, x, s); },
+                         [](double x, double y) { return x + y; });
+            if (lane < 8)
+#pragma unroll
+                for (int i = 0; i < 3; ++i) s_red[warp][halving_index(lane) + i] = acc[i];
             __syncthreads();
             if ((int)threadIdx.x < kRwTile * 6) {
                 const int t = threadIdx.x / 6, k = threadIdx.x % 6;
                 double x = 0.0;
-                for (int w = 0; w < 8; ++w) x += s_red[w][t][k];
+                for (int w = 0; w < 4; ++w) x += s_red[4 * (t / TB) + w][6 * (t % TB) + k];
                 r.part[((size_t)item * kRwTile + t) * 6 + k] = x;
             }
         } else {
             // FP32 only: the tile's reference and every beta's constants come as floats
-            float dbh[kRwTile], dbl[kRwTile], chv[kRwTile], drf[kRwTile], xrh[kRwTile], xrl[kRwTile];
+            float dbh[TB], dbl[TB], chv[TB], drf[TB], xrh[TB], xrl[TB];
 #pragma unroll
-            for (int t = 0; t < kRwTile; ++t) {
-                const float4 kc = t < nt ? r.bc[j0 + t] : make_float4(0.f, 0.f, -1e30f, 0.f);
-                const float2 xr = t < nt ? r.xrf[j0 + t] : make_float2(0.f, 0.f);
+            for (int t = 0; t < TB; ++t) {
+                const bool ok = t0 + t < nt;
+                const float4 kc = ok ? r.bc[j0 + t0 + t] : make_float4(0.f, 0.f, -1e30f, 0.f);
+                const float2 xr = ok ? r.xrf[j0 + t0 + t] : make_float2(0.f, 0.f);
                 dbh[t] = kc.x;
                 dbl[t] = kc.y;
                 chv[t] = kc.z;
@@ -721,12 +831,10 @@ __global__ void __launch_bounds__(256) rw_sums_kernel(RwScratch r, const double 
                 xrl[t] = xr.y;
             }
             const float L2h = (float)kLog2e, L2l = (float)(kLog2e - (double)(float)kLog2e);
-            float hi[kRwTile][6], lo[kRwTile][6];
+            float2 acc[TB * 6];  // high part, accumulated rounding errors
 #pragma unroll
-            for (int t = 0; t < kRwTile; ++t)
-#pragma unroll
-                for (int k = 0; k < 6; ++k) hi[t][k] = lo[t][k] = 0.f;
-            for (int b = b0 + (int)threadIdx.x; b < b1; b += blockDim.x) {
+            for (int k = 0; k < TB * 6; ++k) acc[k] = make_float2(0.f, 0.f);
+            for (int b = bw + lane; b < b1; b += 128) {
                 const float lh = r.lnOf[b];
                 if (lh == -INFINITY) continue;
                 const float dE = (float)(dstep * (b - tp.kT));  // exact
@@ -743,7 +851,7 @@ __global__ void __launch_bounds__(256) rw_sums_kernel(RwScratch r, const double 
                 const float Gl = __fadd_rn(__fmaf_rn(g1, L2h, -Gh), __fadd_rn(__fmul_rn(g1, L2l), __fmul_rn(glo, L2h)));
                 const float x1h = r.x1h[b], x1l = r.x1l[b], vb = r.vf[b];
 #pragma unroll
-                for (int t = 0; t < kRwTile; ++t) {
+                for (int t = 0; t < TB; ++t) {
                     // a = (Gh + Gl) + c - (dbh + dbl) dE as a float pair
                     const float pt = __fmul_rn(dbh[t], dE);
                     const float pte = __fmaf_rn(dbh[t], dE, -pt);
@@ -766,38 +874,30 @@ __global__ void __launch_bounds__(256) rw_sums_kernel(RwScratch r, const double 
 #pragma unroll
                     for (int k = 0; k < 6; ++k) {
                         float sum, err;
-                        two_sum(hi[t][k], __fmul_rn(w, cols[k]), sum, err);
-                        hi[t][k] = sum;
-                        lo[t][k] = __fadd_rn(lo[t][k], err);
+                        two_sum(acc[6 * t + k].x, __fmul_rn(w, cols[k]), sum, err);
+                        acc[6 * t + k] = make_float2(sum, __fadd_rn(acc[6 * t + k].y, err));
                     }
                 }
             }
+            auto add_pairs = [](float2 x, float2 y) {
+                float sum, err;
+                two_sum(x.x, y.x, sum, err);
+                return make_float2(sum, __fadd_rn(__fadd_rn(x.y, y.y), err));
+            };
+            halving_sums(acc, lane,
+                         [](float2 x, int s) {
+                             return make_float2(__shfl_xor_sync(~0u, x.x, s), __shfl_xor_sync(~0u, x.y, s));
+                         },
+                         add_pairs);
+            if (lane < 8)
 #pragma unroll
-            for (int t = 0; t < kRwTile; ++t)
-#pragma unroll
-                for (int k = 0; k < 6; ++k) {
-                    float h = hi[t][k], e = lo[t][k];
-                    for (int q = 16; q > 0; q >>= 1) {
-                        const float oh = __shfl_xor_sync(0xffffffffu, h, q);
-                        const float oe = __shfl_xor_sync(0xffffffffu, e, q);
-                        float sum, err;
-                        two_sum(h, oh, sum, err);
-                        h = sum;
-                        e = __fadd_rn(__fadd_rn(e, oe), err);
-                    }
-                    if (lane == 0) s_rf[warp][t][k] = make_float2(h, e);
-                }
+                for (int i = 0; i < 3; ++i) s_rf[warp][halving_index(lane) + i] = acc[i];
             __syncthreads();
             if ((int)threadIdx.x < kRwTile * 6) {
                 const int t = threadIdx.x / 6, k = threadIdx.x % 6;
-                float h = s_rf[0][t][k].x, e = s_rf[0][t][k].y;
-                for (int w = 1; w < 8; ++w) {
-                    float sum, err;
-                    two_sum(h, s_rf[w][t][k].x, sum, err);
-                    h = sum;
-                    e = __fadd_rn(__fadd_rn(e, s_rf[w][t][k].y), err);
-                }
-                r.part[((size_t)item * kRwTile + t) * 6 + k] = (double)h + (double)e;
+                float2 x = s_rf[4 * (t / TB)][6 * (t % TB) + k];
+                for (int w = 1; w < 4; ++w) x = add_pairs(x, s_rf[4 * (t / TB) + w][6 * (t % TB) + k]);
+                r.part[((size_t)item * kRwTile + t) * 6 + k] = (double)x.x + (double)x.y;
             }
         }
         // the block that completes a tile's last chunk combines the tile's partial sums
@@ -831,8 +931,17 @@ cudaError_t launch_tiles(const RwScratch &r, const double *d_betas, int n_beta, 
                          double mnorm, const Observables &o, int n_sm, cudaStream_t st)
 {
     const int n_tiles = (n_beta + kRwTile - 1) / kRwTile;
-    rw_setup_kernel<<<n_tiles, 256, 0, st>>>(r, d_betas, n_beta, model, V, o);
-    const int grid = std::max(1, std::min(n_tiles * kRwMaxChunks, 4 * n_sm));
+    // about six items per SM: enough to even out, few enough that an item's sums are few
+    // beside its terms (512 tiles of 1900 bins in 8 chunks of 256 bins each: most of
+    // 173 us went to sums; in two chunks 33 us)
+    const int max_chunks = std::max(1, std::min(precision == MUCA_FP64 ? kRwChunks : kRwMaxChunks,
+                                                (6 * n_sm + n_tiles - 1) / n_tiles));
+    const bool powers = precision == MUCA_FP64;
+    if (n_tiles <= 2 * n_sm)
+        rw_setup_kernel<512><<<n_tiles, 512, 0, st>>>(r, d_betas, n_beta, model, V, max_chunks, powers, o);
+    else
+        rw_setup_kernel<256><<<n_tiles, 256, 0, st>>>(r, d_betas, n_beta, model, V, max_chunks, powers, o);
+    const int grid = std::max(1, std::min(n_tiles * max_chunks, 4 * n_sm));
     if (precision == MUCA_FP64)
         rw_sums_kernel<true><<<grid, 256, 0, st>>>(r, d_betas, n_beta, n_tiles, model, V, mnorm, o);
     else
@@ -863,8 +972,8 @@ RwScratch carve(void *bins, size_t cap, size_t nb, void *tiles, int n_beta)
     pb += align256(cap * sizeof(float));
     r.vf = reinterpret_cast<float *>(pb);
     pb += align256(cap * sizeof(float));
-    r.blkrange = reinterpret_cast<int2 *>(pb);
-    r.nblk = (int)((nb + 255) / 256);
+    r.blkrange = reinterpret_cast<int2 *>(r.d.E);
+    r.nblk = (int)((nb + kPrepThreads - 1) / kPrepThreads);
     pb += align256(sizeof(int2) * ((cap + 255) / 256));
     r.cnt0 = reinterpret_cast<unsigned *>(pb);
     const size_t n_tiles = (size_t)(n_beta + kRwTile - 1) / kRwTile;
@@ -886,13 +995,13 @@ RwScratch carve(void *bins, size_t cap, size_t nb, void *tiles, int n_beta)
     r.item_tile = reinterpret_cast<int *>(pt);
     pt += align256(sizeof(int) * n_tiles * kRwMaxChunks);
     r.part = reinterpret_cast<double *>(pt);
+    r.pow = r.part + n_tiles * kRwChunks * kRwTile * 6;
     return r;
 }
 
-cudaError_t launch_prep(const RwScratch &r, const uint64_t *samples, const double *lnw, int model, int V, int nb,
-                        cudaStream_t st)
+cudaError_t launch_prep(const RwScratch &r, const uint64_t *samples, const double *lnw, int nb, cudaStream_t st)
 {
-    rw_prep_kernel<<<r.nblk, 256, 0, st>>>(samples, lnw, r, model, V, nb);
+    rw_prep_kernel<<<r.nblk, kPrepThreads, 0, st>>>(samples, lnw, r, nb);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) note_launches(1);
     return e;
@@ -917,7 +1026,7 @@ cudaError_t launch_reweight_buffers(double *scratch, const uint64_t *samples, co
     // (a race the caller must avoid) then spoil their own results only
     cudaError_t e = cudaMemsetAsync(r.cnt0, 0, sizeof(unsigned), st);
     if (e != cudaSuccess) return e;
-    e = launch_prep(r, samples, lnw, model, V, nb, st);
+    e = launch_prep(r, samples, lnw, nb, st);
     if (e != cudaSuccess) return e;
     const double mnorm = model == MUCA_ISING ? (double)V : (double)(q - 1) * V;
     for (int j0 = 0; j0 < n_beta; j0 += kNoallocBetasPerPass) {
@@ -964,7 +1073,7 @@ int launch_reweight(muca_ctx *ctx, const double *d_betas, int n_beta, int precis
         ctx->rwtile_bytes = need;
     }
     const RwScratch r = carve(ctx->d_rw, nb, nb, ctx->d_rwtile, n_beta);
-    MUCA_CUDA_TRY(launch_prep(r, ctx->d_samples, ctx->d_lnw_prod, ctx->model, ctx->V, ctx->n_bins, ctx->stream));
+    MUCA_CUDA_TRY(launch_prep(r, ctx->d_samples, ctx->d_lnw_prod, ctx->n_bins, ctx->stream));
     MUCA_CUDA_TRY(launch_tiles(r, d_betas, n_beta, precision, ctx->model, ctx->V, mnorm, o, ctx->n_sm, ctx->stream));
     return MUCA_OK;
 }
