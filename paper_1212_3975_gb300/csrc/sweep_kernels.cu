@@ -154,7 +154,7 @@ SweepShape sweep_shape(const muca_ctx *ctx, const SweepPlan &pl, bool hist, int 
     int G = groups;
     if (groups <= 0) {
         double best = 0.0;
-        for (int n = 1; n <= sweep::kMaxGroups; ++n) {
+        for (int n = 1; n <= std::min<long>(sweep::kMaxGroups, all); ++n) {
             if (n > 1 && launch_smem(ctx, pl, hist, staged(n), n, s.lpc) > (size_t)kMaxSmem) break;
             const long waves = ((all + n - 1) / n + ctx->n_sm - 1) / ctx->n_sm;
             const double t = (double)waves * std::max(700.0, 170.0 * n);

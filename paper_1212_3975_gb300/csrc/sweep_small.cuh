@@ -3,10 +3,12 @@
 // A pass of sweep_body.cuh takes a chain of some 600 cycles however few its sites, so on
 // rows of up to 16 sites deciding one site after the other is faster (three iterations of
 // 200 sweeps of 8 x 8 at p = 8, updates included: 2.05 ms with the earlier site-by-site
-// kernel, 2.60 with passes of a row, 1.73 with this body).  The dependent step is kept
+// kernel, 2.60 with passes of a row, 1.43 with this body).  The dependent step is kept
 // short as follows: the table row of the next attempt is one of two candidates (this
 // attempt rejected or accepted), and both candidates' thresholds are loaded before this
-// attempt is decided, so a decision waits for one load and one select.
+// attempt is decided, so a decision waits for one load and one select.  What a row needs at
+// its start (draws, the neighbours of its first sites) is made during the row before: 61
+// cycles per site of 8 x 8 instead of 76, of which some 28 are instructions to issue.
 //
 // A block has G groups of 32 chains: warps 0..G-1 decide, up to four more draw the random
 // numbers into a ring per group (16 sites per hand-off).  Every lane has a histogram of its
@@ -33,28 +35,18 @@ __host__ __device__ constexpr size_t small_smem(int n_bins, int lat_words, int g
     return (size_t)n_bins * 32 + ((hist ? (size_t)n_bins * 128 : 0) + (size_t)lat_words * 128 + SmallRing::kBytes) * groups;
 }
 
-// byte k of x, zero-extended / sign-extended
-__device__ __forceinline__ uint32_t ubyte(uint32_t x, int k)
-{
-    uint32_t d;
-    asm("prmt.b32 %0, %1, 0, %2;" : "=r"(d) : "r"(x), "r"(0x4440u | (uint32_t)k));
-    return d;
-}
-__device__ __forceinline__ uint32_t sbyte(uint32_t x, int k)
-{
-    uint32_t d;
-    asm("prmt.b32 %0, %1, 0, %2;" : "=r"(d) : "r"(x), "r"((uint32_t)k | (8u | (uint32_t)k) * 0x1110u));
-    return d;
-}
-
 // Table offsets 4 n and row changes 64 - 32 n of four sites, one per byte, for the
-// previous attempt rejected (0) / accepted (1); n = unequal neighbours.
+// previous attempt rejected (0) / accepted (1); n = unequal neighbours.  A byte product
+// with 1 in the site's byte adds either to a row address.
 struct Quad {
     uint32_t K0, K1, D0, D1;
 };
 __device__ __forceinline__ Quad quad_of(uint32_t lo, uint32_t hi, uint32_t q, int g)
 {
-    const uint32_t pre = 4u * spread4(lo >> (4 * g)) + 8u * spread4(hi >> (4 * g)), l = 4u * spread4(q >> (4 * g));
+    // (bits 0..3 to bit 2 or 3 of the four bytes)
+    const uint32_t pre = ((((lo >> (4 * g)) & 0xFu) * 0x00810204u) & 0x04040404u) +
+                         ((((hi >> (4 * g)) & 0xFu) * 0x01020408u) & 0x08080808u),
+                   l = (((q >> (4 * g)) & 0xFu) * 0x00810204u) & 0x04040404u;
     Quad r;
     r.K0 = pre + l;
     r.K1 = pre + 0x04040404u - l;
@@ -137,7 +129,7 @@ __device__ __forceinline__ void small_body(const SweepArgs &a, const int cblk, c
         const uint32_t hist0 = (uint32_t)__cvta_generic_to_shared(s_hist + 32 * n_bins * grp + lane) - 4u * tab0;
 
         // P0 / P1: table row before the site if the previous attempt was rejected / accepted
-        // (ap: which); D0 / D1: its change if the site accepts, A0 / A1: the thresholds
+        // (ap: which); Q0 / Q1: the row after it if the site accepts, A0 / A1: the thresholds
         uint32_t P0 = tab0 + 32u * (uint32_t)(active ? (a.E[c] + 2 * V) >> 2 : V >> 1), P1 = P0;
         bool ap = false;
         uint32_t R = row_of(0), U = row_of(L - 1), D = row_of(1);
@@ -147,64 +139,80 @@ __device__ __forceinline__ void small_body(const SweepArgs &a, const int cblk, c
             return ((s ^ u) & 1u) + ((s ^ d) & 1u) + ((s ^ (r >> 1)) & 1u) + ((s ^ (r >> (L - 1))) & 1u);
         };
         const uint32_t n = first_site(R, U, D);
-        uint32_t D0 = 64u - 32u * n, D1 = D0;
+        uint32_t Q0 = P0 + 64u - 32u * n, Q1 = Q0;
         uint32_t A0 = lds32(P0 + 4u * n), A1 = A0;
-        bar_sync(1 + grp, 64);
         const int rows = a.n_sweeps * L;
         int y = 0, sw = 0, pos = 0, lin = L, next_sync = Rg::kPhase;
         int ups = 0;
+        // draws of the row; each block of four (two) makes room for the next row's
+        uint32_t u[L];
+        constexpr int W = L % 4 == 0 ? 4 : 2;
+        auto load_draws = [&](int j) {
+            const uint32_t us = ring_s + 4u * (uint32_t)(pos + j);
+            if constexpr (W == 4)
+                asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                             : "=r"(u[j]), "=r"(u[j + 1]), "=r"(u[j + 2]), "=r"(u[j + 3])
+                             : "r"(us));
+            else
+                asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(u[j]), "=r"(u[j + 1]) : "r"(us));
+        };
+        auto next_draws = [&] {
+            pos = pos + L >= Rg::kSites ? pos + L - Rg::kSites : pos + L;
+            lin += L;
+        };
+        bar_sync(1 + grp, 64);
+#pragma unroll
+        for (int j = 0; j < L; j += W) load_draws(j);
+        next_draws();
+        Quad qd;  // of the four sites around the next one
+        {
+            const uint32_t ua = R ^ U, ub = R ^ D, tr = R ^ (R >> 1);
+            qd = quad_of(ua ^ ub ^ tr, (ua & ub) | (tr & (ua ^ ub)), R ^ (R << 1), 0);
+        }
         for (int it = 0; it < rows; ++it) {
-            // the row's draws are handed off
+            // the next row's draws are handed off (past the last row: old ones, not used)
             if (lin > next_sync) {
                 if (next_sync < phases * Rg::kPhase) bar_sync(1 + grp, 64);
                 next_sync += Rg::kPhase;
             }
-            const uint32_t us = ring_s + 4u * (uint32_t)pos;
-            uint32_t u[L];
-            if constexpr (L % 4 == 0) {
-#pragma unroll
-                for (int j = 0; j < L; j += 4)
-                    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                                 : "=r"(u[j]), "=r"(u[j + 1]), "=r"(u[j + 2]), "=r"(u[j + 3])
-                                 : "r"(us + 4u * j));
-            } else {
-#pragma unroll
-                for (int j = 0; j < L; j += 2)
-                    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(u[j]), "=r"(u[j + 1]) : "r"(us + 4u * j));
-            }
-            pos = pos + L >= Rg::kSites ? pos + L - Rg::kSites : pos + L;
-            lin += L;
             const int y1 = y + 1 == L ? 0 : y + 1;
             const uint32_t R1 = row_of(y1), D1w = row_of(y1 + 1 == L ? 0 : y1 + 1);
             const uint32_t ua = R ^ U, ub = R ^ D, tr = R ^ (R >> 1), q = R ^ (R << 1);
             const uint32_t lo = ua ^ ub ^ tr, hi = (ua & ub) | (tr & (ua ^ ub));
             uint32_t Rw = R, last = 0u;  // last: unequal neighbours of the last site but its left one
-            Quad qd = quad_of(lo, hi, q, 0);
+            uint32_t n1 = 0u;                // unequal neighbours of the next row's first site
+            Quad qn;                         // the next row's first quad
 #pragma unroll
             for (int j = 0; j < L; ++j) {
+                // (what the next row needs of this one's first sites, as soon as these are
+                // decided: the row's end does not wait for it)
+                if (j == 1) n1 = first_site(R1, Rw, D1w);
+                if (L >= 6 && j == L - 2) {
+                    const uint32_t va = R1 ^ Rw, vb = R1 ^ D1w, tr1 = R1 ^ (R1 >> 1);
+                    qn = quad_of(va ^ vb ^ tr1, (va & vb) | (tr1 & (va ^ vb)), R1 ^ (R1 << 1), 0);
+                }
                 // the next site's table offset and row change, for this attempt rejected / accepted
-                uint32_t K0, K1, E0, E1;
+                const uint32_t Pc = ap ? P1 : P0, Pa = ap ? Q1 : Q0;
+                uint32_t B0, B1;
                 if (j + 1 == L) {
-                    // (of the row below only site 0 is needed yet: its upper neighbour is decided)
-                    const uint32_t n1 = first_site(R1, Rw, D1w);
-                    K0 = K1 = 4u * n1;
-                    E0 = E1 = 64u - 32u * n1;
+                    B0 = lds32(Pc + 4u * n1);
+                    B1 = lds32(Pa + 4u * n1);
+                    Q0 = Pc + 64u - 32u * n1;
+                    Q1 = Pa + 64u - 32u * n1;
                 } else if (j + 2 == L) {
-                    const uint32_t l = (q >> (L - 1)) & 1u;
-                    K0 = 4u * (last + l);
-                    K1 = 4u * (last + 1u - l);
-                    E0 = 64u - 8u * K0;
-                    E1 = 64u - 8u * K1;
+                    const uint32_t l = (q >> (L - 1)) & 1u, k0 = last + l, k1 = last + 1u - l;
+                    B0 = lds32(Pc + 4u * k0);
+                    B1 = lds32(Pa + 4u * k1);
+                    Q0 = Pc + 64u - 32u * k0;
+                    Q1 = Pa + 64u - 32u * k1;
                 } else {
                     if ((j & 3) == 3) qd = quad_of(lo, hi, q, (j + 1) >> 2);
-                    const int k = (j + 1) & 3;
-                    K0 = ubyte(qd.K0, k);
-                    K1 = ubyte(qd.K1, k);
-                    E0 = sbyte(qd.D0, k);
-                    E1 = sbyte(qd.D1, k);
+                    const int k = 1 << (8 * ((j + 1) & 3));
+                    B0 = lds32((uint32_t)__dp4a((int)qd.K0, k, (int)Pc));
+                    B1 = lds32((uint32_t)__dp4a((int)qd.K1, k, (int)Pa));
+                    Q0 = (uint32_t)__dp4a((int)qd.D0, k, (int)Pc);
+                    Q1 = (uint32_t)__dp4a((int)qd.D1, k, (int)Pa);
                 }
-                const uint32_t Pc = ap ? P1 : P0, Pa = Pc + (ap ? D1 : D0);
-                const uint32_t B0 = lds32(Pc + K0), B1 = lds32(Pa + K1);
                 const bool acc = u[j] < (ap ? A1 : A0);
                 if (HIST) red_shared(hist0 + 4u * (acc ? Pa : Pc), 1u);
                 Rw ^= acc ? 1u << j : 0u;
@@ -212,12 +220,12 @@ __device__ __forceinline__ void small_body(const SweepArgs &a, const int cblk, c
                     last = ((ua >> (L - 1)) & 1u) + ((ub >> (L - 1)) & 1u) + (((R >> (L - 1)) ^ Rw) & 1u);
                 P0 = Pc;
                 P1 = Pa;
-                D0 = E0;
-                D1 = E1;
                 A0 = B0;
                 A1 = B1;
                 ap = acc;
+                if (j % W == W - 1) load_draws(j - (W - 1));
             }
+            next_draws();
             asm volatile("st.shared.u32 [%0], %1;" ::"r"(lat_s + (uint32_t)y * ls), "r"(Rw) : "memory");
             ups += __popc(Rw);
             if (y1 == 0) {
@@ -237,6 +245,11 @@ __device__ __forceinline__ void small_body(const SweepArgs &a, const int cblk, c
                 if (it + 1 < rows) ups = 0;
             }
             // (R1 and D1w were read before this row was stored: at L >= 4 they are other rows)
+            if (L < 6) {
+                const uint32_t va = R1 ^ Rw, vb = R1 ^ D1w, tr1 = R1 ^ (R1 >> 1);
+                qn = quad_of(va ^ vb ^ tr1, (va & vb) | (tr1 & (va ^ vb)), R1 ^ (R1 << 1), 0);
+            }
+            qd = qn;
             U = Rw;
             R = R1;
             D = D1w;
