@@ -72,59 +72,68 @@ struct BlockStats {
 // The update runs as two kernels.  The recursion's differences (two logarithms and two
 // divisions in FP64 per bin, at two FP64 operations per clock and SM: 0.15 ms for 4097
 // bins on one SM) take a grid of blocks; what follows is one block per lattice
-// (blockDim.x = 1024):
+// (kUpdateThreads):
 //   1. convergence statistics of H over accessible bins (Sec. 3);
 //   2. prefix sums of the differences over accessible bins in ascending order, rounded
 //      as the sequential sum (prefix_piece);
 //   3. boundary correction beyond [lo, hi] with the slope of the innermost
 //      `width` bins (Sec. 3);
 //   4. ln W -= max over accessible bins; inaccessible bins = 0.
-constexpr int kPiece = 4096;  // bins of the prefix staged at a time
+constexpr int kPiece = 4096;         // bins of the prefix staged at a time
+constexpr int kPrefixThreads = 256;  // threads of the prefix, four bins each at a time
 
-// Sequential FP64 sum cur += x[i] of n values in shared memory, in place, by one warp, 128
-// values at a time; returns the last sum.  The result is that of adding one value after
-// the other, bit for bit: while the sum stays in one binade it is a multiple k of one unit
-// u in the last place, and adding x rounds to k + (x / u rounded to the nearest integer),
-// so a run of additions is a prefix sum of integers.  Where that does not hold (a sum that
-// leaves the binade or changes sign, an x / u halfway between integers, an x above the
-// binade, a sum of zero) the one addition is done in FP64.  A chain of FP64 additions takes
-// 117 cycles per value on this GPU (two FP64 operations per clock and SM): 0.23 ms for the
-// 4097 bins of a 64 x 64 Ising lattice, 0.93 ms for 128 x 128, against 0.01 ms and 0.04 ms.
-__device__ __forceinline__ double prefix_piece(double *x, int n, double cur, int lane)
+__device__ __forceinline__ void prefix_barrier()
+{
+    asm volatile("bar.sync 1, %0;" ::"n"(kPrefixThreads) : "memory");
+}
+
+// Sequential FP64 sum cur += x[i] of n values in shared memory, in place, by the block's
+// first kPrefixThreads threads, four values each at a time; returns the last sum.  The
+// result is that of adding one value after the other, bit for bit: while the sum stays in
+// one binade it is a multiple k of one unit u in the last place, and adding x rounds to
+// k + (x / u rounded to the nearest integer), so a run of additions is a prefix sum of
+// integers.  Where that does not hold (a sum that leaves the binade or changes sign, an
+// x / u halfway between integers, an x above the binade, a sum of zero) the one addition is
+// done in FP64.  A chain of FP64 additions takes 117 cycles per value on this GPU (two FP64
+// operations per clock and SM): 0.23 ms for the 4097 bins of a 64 x 64 Ising lattice.  One
+// warp took 50 rounds of 128 values at 1750 cycles each for 64 x 64
+// (18 of them for sums that leave their binade); with eight warps and
+// rounds of 1024 values the whole update kernel takes 40 us instead of 68 (90 x 90: 64
+// instead of 105).
+__device__ __forceinline__ double prefix_piece(double *x, int n, double cur, int tid)
 {
     constexpr unsigned long long one = 1ull << 52, frac = one - 1ull;
+    constexpr int NW = kPrefixThreads / 32, span = 4 * kPrefixThreads;
+    __shared__ long long s_tot[NW];
+    __shared__ int s_stop[NW];
+    const int lane = tid & 31, warp = tid >> 5;
+    int late = -1;  // a sum still to be stored (thread 0)
+    double late_sum = 0.0;
     for (int i = 0; i < n;) {
         const unsigned long long cb = (unsigned long long)__double_as_longlong(cur);
         const int ce = (int)(cb >> 52) & 0x7FF;
         const long long mag = (long long)((cb & frac) | one), k = cb >> 63 ? -mag : mag;
         const bool zero = cb == 0ull, regular = ce > 0 && ce < 0x7FF;
-        long long v[4];   // the lane's inclusive sums of rounded integers
-        int good = 4;     // values of the lane before the first that needs FP64
+        long long v[4];   // the thread's inclusive sums of rounded integers
+        int good = 4;     // values of the thread before the first that needs FP64
         long long sum = 0;
+        const int j0 = i + 4 * tid;
+#pragma unroll
+        for (int t = 3; t >= 0; --t) v[t] = __double_as_longlong(j0 + t < n ? x[j0 + t] : 0.0);
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
-            const int j = i + 4 * lane + t;
-            bool ok = j < n && (regular || zero);
-            if (ok) {
-                const unsigned long long b = (unsigned long long)__double_as_longlong(x[j]);
-                if (zero) {
-                    ok = (b << 1) == 0ull;
-                } else {
-                    int e = (int)(b >> 52) & 0x7FF;
-                    const unsigned long long mt = (b & frac) | (e ? one : 0ull);
-                    const int sh = ce - (e ? e : 1);
-                    ok = e != 0x7FF && sh >= 0;
-                    if (ok && sh <= 54) {
-                        const unsigned long long half = sh ? 1ull << (sh - 1) : 0ull;
-                        const unsigned long long low = sh ? mt & ((half << 1) - 1ull) : 0ull;
-                        ok = !(sh && low == half);
-                        const long long r = (long long)((mt + half) >> sh);
-                        sum += b >> 63 ? -r : r;
-                    }
-                }
-            }
-            v[t] = sum;
+            const unsigned long long b = (unsigned long long)v[t];
+            const int e = (int)(b >> 52) & 0x7FF, sh = ce - max(e, 1);
+            const unsigned long long mt = ((b & frac) | (e ? one : 0ull)) << 1;
+            // x / u with one more bit, and whether that is all of it
+            const int s = min(max(sh, 0), 63);
+            const unsigned long long r2 = mt >> s;
+            const bool tie = (r2 & 1ull) && (r2 << s) == mt;
+            const long long r = (long long)((r2 + 1ull) >> 1);
+            const bool ok = j0 + t < n && (zero ? (b << 1) == 0ull : regular && e != 0x7FF && sh >= 0 && !tie);
             if (!ok) good = min(good, t);
+            if (!zero) sum += b >> 63 ? -r : r;
+            v[t] = sum;
         }
         long long incl = sum;
 #pragma unroll
@@ -132,37 +141,53 @@ __device__ __forceinline__ double prefix_piece(double *x, int n, double cur, int
             const long long y = __shfl_up_sync(~0u, incl, o);
             if (lane >= o) incl += y;
         }
-        const long long below = k + incl - sum;
+        if (lane == 31) s_tot[warp] = incl;
+        prefix_barrier();
+        if (late >= 0 && tid == 0) x[late] = late_sum;
+        long long below = k + incl - sum;
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
+        for (int w = 0; w < NW - 1; ++w)
+            if (w < warp) below += s_tot[w];
+#pragma unroll
+        for (int t = 3; t >= 0; --t) {
             v[t] += below;
             const unsigned long long q = (unsigned long long)(v[t] < 0 ? -v[t] : v[t]);
             if (!zero && !(q > one && q < one << 1 && (v[t] < 0) == (k < 0))) good = min(good, t);
         }
-        const unsigned stop = __ballot_sync(~0u, good < 4);
-        const int first = stop ? __ffs(stop) - 1 : 32;
-        const int done = stop ? 4 * first + __shfl_sync(~0u, good, first & 31) : 128;  // (values past n stop it)
+        const int stop = __reduce_min_sync(~0u, good < 4 ? 4 * tid + good : span);
+        if (lane == 0) s_stop[warp] = stop;
+        prefix_barrier();
+        int done = s_stop[0];  // (values past n stop it)
+#pragma unroll
+        for (int w = 1; w < NW; ++w) done = min(done, s_stop[w]);
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
-            if (4 * lane + t < done) {
+            if (4 * tid + t < done) {
                 const unsigned long long q = (unsigned long long)(v[t] < 0 ? -v[t] : v[t]);
                 const unsigned long long bits = zero ? 0ull : (q & frac) | (unsigned long long)ce << 52 | (cb & (1ull << 63));
-                x[i + 4 * lane + t] = __longlong_as_double((long long)bits);
+                x[j0 + t] = __longlong_as_double((long long)bits);
             }
         }
-        __syncwarp();
+        prefix_barrier();
         if (done > 0) cur = x[i + done - 1];
         i += done;
-        if (done < 128 && i < n) {
+        late = -1;
+        if (done < span && i < n) {
+            // (stored when every thread has read it)
             cur = __dadd_rn(cur, x[i]);
-            __syncwarp();
-            if (lane == 0) x[i] = cur;
+            late = i;
+            late_sum = cur;
             ++i;
         }
-        __syncwarp();
     }
+    prefix_barrier();
+    if (late >= 0 && tid == 0) x[late] = late_sum;
     return cur;
 }
+
+// Threads per block where every thread evaluates FP64 logarithms, divisions or an
+// exponential: small, so that the bins spread over all SMs' FP64 pipes.
+constexpr int kBinThreads = 64;
 
 // Recursion (Sec. 2) of bin u: scratch[v] = difference to bin v from the accessible bin u
 // before it (accumulated form), or ln W after the simple recursion.
@@ -192,133 +217,147 @@ __device__ __forceinline__ void update_bin(const double *lnw, double *P, double 
     }
 }
 
+// Order of doubles as integers (NaN lowest): the FP64 maximum of a block is 32 comparisons
+// in a row at some 100 cycles each.
+__device__ __forceinline__ long long order_key(double x)
+{
+    const long long b = __double_as_longlong(x);
+    return x != x ? (long long)(1ull << 63) : b < 0 ? b ^ 0x7FFFFFFFFFFFFFFFll : b;
+}
+__device__ __forceinline__ double order_value(long long k)
+{
+    return __longlong_as_double(k < 0 ? k ^ 0x7FFFFFFFFFFFFFFFll : k);
+}
+
+// blockDim.x = kUpdateThreads
+constexpr int kUpdateThreads = 1024;
 __device__ __forceinline__ void update_body(double *lnw, const double *scratch, const uint64_t *H, const uint8_t *acc,
                                             int n_bins, int accumulated, int width_cfg, muca_iter_stats *stats)
 {
-    __shared__ unsigned long long s_total[32], s_min[32], s_max[32], s_ns[32], s_K[32];
-    __shared__ int s_lo[32], s_hi[32];
-    __shared__ double s_top[32];
-    __shared__ int sh_lo, sh_hi;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    constexpr int NW = kUpdateThreads / 32;
+    static_assert(NW == 32, "a warp reduces the warps' values");
+    __shared__ unsigned long long s_total[NW], s_min[NW], s_max[NW];
+    __shared__ int s_ns[NW], s_K[NW], s_lo[NW], s_hi[NW], s_first[NW];
+    __shared__ long long s_top[NW];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
     // 1. statistics
-    unsigned long long tot = 0, mn = ~0ull, mx = 0, ns = 0, K = 0;
-    int lo = n_bins, hi = -1;
-    for (int b = tid; b < n_bins; b += blockDim.x) {
+    unsigned long long tot = 0, mn = ~0ull, mx = 0;
+    int ns = 0, K = 0, lo = n_bins, hi = -1, first = n_bins;
+    for (int b = tid; b < n_bins; b += kUpdateThreads) {
         if (!acc[b]) continue;
         const unsigned long long h = H[b];
         tot += h;
         mn = min(mn, h);
         mx = max(mx, h);
         K += 1;
+        first = min(first, b);
         if (h) {
             ns += 1;
             lo = min(lo, b);
             hi = max(hi, b);
         }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        tot += __shfl_xor_sync(0xffffffffu, tot, o);
-        mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        ns += __shfl_xor_sync(0xffffffffu, ns, o);
-        K += __shfl_xor_sync(0xffffffffu, K, o);
-        lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-        hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-    }
+    auto reduce_counts = [&] {
+        for (int o = 16; o > 0; o >>= 1) {
+            tot += __shfl_xor_sync(~0u, tot, o);
+            mn = min(mn, __shfl_xor_sync(~0u, mn, o));
+            mx = max(mx, __shfl_xor_sync(~0u, mx, o));
+        }
+        ns = __reduce_add_sync(~0u, ns);
+        K = __reduce_add_sync(~0u, K);
+    };
+    reduce_counts();
+    lo = __reduce_min_sync(~0u, lo);
+    hi = __reduce_max_sync(~0u, hi);
+    first = __reduce_min_sync(~0u, first);
     if (lane == 0) {
         s_total[warp] = tot; s_min[warp] = mn; s_max[warp] = mx; s_ns[warp] = ns; s_K[warp] = K;
-        s_lo[warp] = lo; s_hi[warp] = hi;
+        s_lo[warp] = lo; s_hi[warp] = hi; s_first[warp] = first;
     }
     __syncthreads();
-    if (tid == 0) {
-        for (int w = 1; w < nw; ++w) {
-            tot += s_total[w]; mn = min(mn, s_min[w]); mx = max(mx, s_max[w]); ns += s_ns[w]; K += s_K[w];
-            lo = min(lo, s_lo[w]); hi = max(hi, s_hi[w]);
+    lo = __reduce_min_sync(~0u, s_lo[lane]);
+    hi = __reduce_max_sync(~0u, s_hi[lane]);
+    first = __reduce_min_sync(~0u, s_first[lane]);
+    const int slo = hi >= 0 ? lo : -1, shi = hi >= 0 ? hi : -1;
+    if (warp == NW - 1) {
+        // (beside the prefix: five FP64 divisions and comparisons in a row)
+        tot = s_total[lane]; mn = s_min[lane]; mx = s_max[lane]; ns = s_ns[lane]; K = s_K[lane];
+        reduce_counts();
+        if (lane == 0) {
+            const double mean = (double)tot / (double)(unsigned long long)K;
+            muca_iter_stats st;
+            st.covered = (ns == K);
+            st.flat = st.covered && ((double)mn >= 0.5 * mean) && ((double)mx <= 2.0 * mean);
+            st.lo = slo;
+            st.hi = shi;
+            st.n_sampled = (int64_t)ns;
+            st.min_over_mean = mean > 0 ? (double)mn / mean : 0.0;
+            st.max_over_mean = mean > 0 ? (double)mx / mean : 0.0;
+            st.total = tot;
+            *stats = st;
         }
-        const double mean = (double)tot / (double)K;
-        muca_iter_stats st;
-        st.covered = (ns == K);
-        st.flat = st.covered && ((double)mn >= 0.5 * mean) && ((double)mx <= 2.0 * mean);
-        st.lo = hi >= 0 ? lo : -1;
-        st.hi = hi >= 0 ? hi : -1;
-        st.n_sampled = (int64_t)ns;
-        st.min_over_mean = mean > 0 ? (double)mn / mean : 0.0;
-        st.max_over_mean = mean > 0 ? (double)mx / mean : 0.0;
-        st.total = tot;
-        *stats = st;
-        sh_lo = st.lo;
-        sh_hi = st.hi;
     }
-    __syncthreads();
 
     // 2. prefix in ascending order
     if (accumulated) {
         __shared__ double s_d[kPiece];
-        __shared__ int s_first;
-        if (tid == 0) {
-            int u = 0;
-            while (!acc[u]) ++u;
-            s_first = u;
-        }
-        double cur = 0.0;  // (warp 0)
+        double cur = 0.0;  // (threads of the prefix)
         for (int b0 = 0; b0 < n_bins; b0 += kPiece) {
             const int n = min(kPiece, n_bins - b0);
-            __syncthreads();
             // (an inaccessible bin adds nothing; the first accessible one has no difference)
-            for (int i = tid; i < n; i += blockDim.x)
-                s_d[i] = acc[b0 + i] && b0 + i != s_first ? scratch[b0 + i] : 0.0;
+            for (int i = tid; i < n; i += kUpdateThreads)
+                s_d[i] = acc[b0 + i] && b0 + i != first ? scratch[b0 + i] : 0.0;
             __syncthreads();
-            if (warp == 0) cur = prefix_piece(s_d, n, cur, lane);
+            if (tid < kPrefixThreads) cur = prefix_piece(s_d, n, cur, tid);
             __syncthreads();
-            for (int i = tid; i < n; i += blockDim.x)
+            for (int i = tid; i < n; i += kUpdateThreads)
                 if (acc[b0 + i]) lnw[b0 + i] = s_d[i];
             __syncthreads();
         }
     } else {
-        for (int b = tid; b < n_bins; b += blockDim.x)
+        for (int b = tid; b < n_bins; b += kUpdateThreads)
             if (acc[b]) lnw[b] = scratch[b];
+        __syncthreads();
     }
-    __syncthreads();
 
     // 3. boundary correction
-    const int slo = sh_lo, shi = sh_hi;
-    if (slo >= 0 && shi > slo) {
+    const bool bounds = slo >= 0 && shi > slo;
+    double vlo = 0.0, vhi = 0.0;
+    __shared__ double s_slope[2];
+    if (bounds) {
         const int width = min(width_cfg, shi - slo);
-        __shared__ double sl_lo, sl_hi;
-        if (tid == 0) {
-            int b2 = slo + width;
-            while (!acc[b2]) ++b2;
-            int b1 = shi - width;
-            while (!acc[b1]) --b1;
-            sl_lo = __ddiv_rn(__dsub_rn(lnw[b2], lnw[slo]), (double)(b2 - slo));
-            sl_hi = __ddiv_rn(__dsub_rn(lnw[shi], lnw[b1]), (double)(shi - b1));
+        if (lane == 0 && warp < 2) {
+            // (warp 0 the lower, warp 1 the upper end)
+            int b = warp == 0 ? slo + width : shi - width;
+            while (!acc[b]) b += warp == 0 ? 1 : -1;
+            s_slope[warp] = warp == 0 ? __ddiv_rn(__dsub_rn(lnw[b], lnw[slo]), (double)(b - slo))
+                                      : __ddiv_rn(__dsub_rn(lnw[shi], lnw[b]), (double)(shi - b));
         }
+        vlo = lnw[slo];
+        vhi = lnw[shi];
         __syncthreads();
-        const double vlo = lnw[slo], vhi = lnw[shi];
-        __syncthreads();
-        for (int b = tid; b < n_bins; b += blockDim.x) {
-            if (!acc[b]) continue;
-            if (b < slo) lnw[b] = __dadd_rn(vlo, __dmul_rn(sl_lo, (double)(b - slo)));
-            else if (b > shi) lnw[b] = __dadd_rn(vhi, __dmul_rn(sl_hi, (double)(b - shi)));
-        }
     }
-    __syncthreads();
+    const double sl_lo = s_slope[0], sl_hi = s_slope[1];
 
     // 4. normalisation: max over accessible bins is 0
-    double top = -INFINITY;
-    for (int b = tid; b < n_bins; b += blockDim.x)
-        if (acc[b]) top = fmax(top, lnw[b]);
-    for (int o = 16; o > 0; o >>= 1) top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
-    if (lane == 0) s_top[warp] = top;
-    __syncthreads();
-    if (tid == 0) {
-        for (int w = 1; w < nw; ++w) top = fmax(top, s_top[w]);
-        s_top[0] = top;
+    long long key = (long long)(1ull << 63);
+    for (int b = tid; b < n_bins; b += kUpdateThreads) {
+        if (!acc[b]) continue;
+        double x;
+        if (bounds && b < slo) x = lnw[b] = __dadd_rn(vlo, __dmul_rn(sl_lo, (double)(b - slo)));
+        else if (bounds && b > shi) x = lnw[b] = __dadd_rn(vhi, __dmul_rn(sl_hi, (double)(b - shi)));
+        else x = lnw[b];
+        key = max(key, order_key(x));
     }
+    for (int o = 16; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(~0u, key, o));
+    if (lane == 0) s_top[warp] = key;
     __syncthreads();
-    top = s_top[0];
-    for (int b = tid; b < n_bins; b += blockDim.x) lnw[b] = acc[b] ? __dsub_rn(lnw[b], top) : 0.0;
+    key = s_top[lane];
+    for (int o = 16; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(~0u, key, o));
+    const double top = order_value(key);
+    // (each bin was last written by its own thread)
+    for (int b = tid; b < n_bins; b += kUpdateThreads) lnw[b] = acc[b] ? __dsub_rn(lnw[b], top) : 0.0;
 }
 
 __global__ void update_bins_kernel(const double *lnw, double *P, double *scratch, const uint64_t *H, const uint8_t *acc,
@@ -328,7 +367,7 @@ __global__ void update_bins_kernel(const double *lnw, double *P, double *scratch
     if (u < n_bins) update_bin(lnw, P, scratch, H, acc, n_bins, accumulated, u);
 }
 
-__global__ void __launch_bounds__(1024) update_kernel(double *lnw, const double *scratch, const uint64_t *H,
+__global__ void __launch_bounds__(kUpdateThreads) update_kernel(double *lnw, const double *scratch, const uint64_t *H,
                                                       const uint8_t *acc, int n_bins, int accumulated, int width_cfg,
                                                       muca_iter_stats *stats)
 {
@@ -344,7 +383,7 @@ __global__ void update_bins_batch_kernel(const BatchJob *jobs)
     if (u < j.n_bins) update_bin(j.lnw, j.P, j.wscratch, j.H, j.acc, j.n_bins, j.accumulated, u);
 }
 
-__global__ void __launch_bounds__(1024) update_batch_kernel(const BatchJob *jobs)
+__global__ void __launch_bounds__(kUpdateThreads) update_batch_kernel(const BatchJob *jobs)
 {
     const BatchJob &j = jobs[blockIdx.x];
     if (!*j.active) return;
@@ -377,14 +416,14 @@ __global__ void thresholds_batch_kernel(const BatchJob *jobs)
 
 cudaError_t launch_batch_update(const BatchJob *d_jobs, int n_jobs, int max_bins, int max_thr, cudaStream_t st)
 {
-    update_bins_batch_kernel<<<dim3((max_bins + 127) / 128, n_jobs), 128, 0, st>>>(d_jobs);
+    update_bins_batch_kernel<<<dim3((max_bins + kBinThreads - 1) / kBinThreads, n_jobs), kBinThreads, 0, st>>>(d_jobs);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    update_batch_kernel<<<n_jobs, 1024, 0, st>>>(d_jobs);
+    update_batch_kernel<<<n_jobs, kUpdateThreads, 0, st>>>(d_jobs);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    dim3 grid((max_thr + 255) / 256, n_jobs);
-    thresholds_batch_kernel<<<grid, 256, 0, st>>>(d_jobs);
+    dim3 grid((max_thr + kBinThreads - 1) / kBinThreads, n_jobs);
+    thresholds_batch_kernel<<<grid, kBinThreads, 0, st>>>(d_jobs);
     e = cudaGetLastError();
     if (e == cudaSuccess) note_launches(3);
     return e;
@@ -394,8 +433,8 @@ int launch_thresholds(muca_ctx *ctx)
 {
     if (ctx->cfg.ensemble == MUCA_ENSEMBLE_MAGNETIZATION) return launch_muma_thresholds(ctx);
     const int n = ctx->n_bins * ctx->n_de;
-    thresholds_kernel<<<(n + 255) / 256, 256, 0, ctx->stream>>>(ctx->d_lnw, ctx->d_acc, ctx->d_thr, ctx->model,
-                                                               ctx->n_bins, ctx->n_de);
+    thresholds_kernel<<<(n + kBinThreads - 1) / kBinThreads, kBinThreads, 0, ctx->stream>>>(
+        ctx->d_lnw, ctx->d_acc, ctx->d_thr, ctx->model, ctx->n_bins, ctx->n_de);
     MUCA_CUDA_TRY(cudaGetLastError());
     note_launches(1);
     ctx->ktab_dirty = 1;
@@ -406,11 +445,11 @@ int launch_update(muca_ctx *ctx)
 {
     const int width = ctx->cfg.correction_width > 0 ? ctx->cfg.correction_width : ctx->L;
     const int accumulated = ctx->cfg.recursion == MUCA_RECURSION_ACCUMULATED;
-    update_bins_kernel<<<(ctx->n_bins + 127) / 128, 128, 0, ctx->stream>>>(ctx->d_lnw, ctx->d_P, ctx->d_wscratch, ctx->d_H,
-                                                                          ctx->d_acc, ctx->n_bins, accumulated);
+    update_bins_kernel<<<(ctx->n_bins + kBinThreads - 1) / kBinThreads, kBinThreads, 0, ctx->stream>>>(
+        ctx->d_lnw, ctx->d_P, ctx->d_wscratch, ctx->d_H, ctx->d_acc, ctx->n_bins, accumulated);
     MUCA_CUDA_TRY(cudaGetLastError());
-    update_kernel<<<1, 1024, 0, ctx->stream>>>(ctx->d_lnw, ctx->d_wscratch, ctx->d_H, ctx->d_acc, ctx->n_bins, accumulated,
-                                               width, ctx->d_stats);
+    update_kernel<<<1, kUpdateThreads, 0, ctx->stream>>>(ctx->d_lnw, ctx->d_wscratch, ctx->d_H, ctx->d_acc, ctx->n_bins,
+                                                         accumulated, width, ctx->d_stats);
     MUCA_CUDA_TRY(cudaGetLastError());
     note_launches(2);
     return launch_thresholds(ctx);
