@@ -38,6 +38,8 @@
 // signs are combined with logic instructions (5 cycles a step, a predicate takes 13).  A
 // difference of zero leaves the test open (once in 2^31): the 32-bit table decides it.
 #pragma once
+#include <type_traits>
+
 #include "muca_internal.cuh"
 
 namespace muca {
@@ -72,6 +74,12 @@ __host__ __device__ constexpr size_t ring_bytes(int model) { return 6656 + (mode
 __device__ __forceinline__ void bar_sync(int id, int n)
 {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+// the same where `take` is true (uniform): no branch
+__device__ __forceinline__ void bar_sync_if(bool take, int id, int n)
+{
+    asm volatile("{.reg .pred p; setp.ne.u32 p, %2, 0; @p bar.sync %0, %1;}" ::"r"(id), "r"(n), "r"((uint32_t)take)
+                 : "memory");
 }
 __device__ __forceinline__ void red_shared(uint32_t saddr, uint32_t v)
 {
@@ -184,7 +192,10 @@ struct StateCounts {
 // that a branch would decide in every pass, are template parameters: with one deciding
 // warp per scheduler a uniform branch costs a pass some 20 cycles (64 x 64, p = 1024: 566
 // against 375 ns per pass with the modes as run-time flags).
-template <int MODEL, int LPC, bool ROW, bool AL, int TAB, int HMODE>
+// PEEL: the first attempt of a pass is code of its own, in whose gaps the next pass is
+// prepared, and a repetition does without that.  Shorter passes while latency bounds them,
+// more code than the instruction caches like where a scheduler has three deciding warps.
+template <int MODEL, int LPC, bool ROW, bool AL, int TAB, int HMODE, bool PEEL>
 __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, const int G, const bool stage_lattice,
                                            uint32_t *smem)
 {
@@ -198,6 +209,7 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
     constexpr uint32_t m = 0x01010101u;
     constexpr bool HIST = HMODE != kHistNone;
     static_assert(ROW || LPC == 32, "long rows take whole warps");
+    static_assert(ROW || !PEEL, "rows of one pass");
     static_assert(AL || HMODE != kHistPairs, "pairs lie within a lane's four sites");
     __syncthreads();  // (persistent kernel: smem may still be read by the previous unit)
     const int tid = threadIdx.x, nt = block_threads(G), lane = tid & 31, warp = tid >> 5;
@@ -253,7 +265,7 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                 const int d0 = slot * Rg::kPhase + 4 * cl;
                 qd = qd0;
                 ctr1 = ctr0;
-#pragma unroll(POTTS ? 2 : 4)
+#pragma unroll 2
                 for (int pass = 0; pass < 4; ++pass) {
                     uint4 b;
                     uint32_t off = 0u;
@@ -476,15 +488,20 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
             const int skip = !AL && lastq && last_row ? VS - V : 0;
             int pos1 = pos + len + skip;
             pos1 = pos1 >= Rg::kSites ? pos1 - Rg::kSites : pos1;
-            ahead -= skip + len1;
-            if (ahead < 0) {
-                if (taken < phases) bar_sync(1 + grp, 64);
-                ++taken;
-                ahead += Rg::kPhase;
-            }
-            if (POTTS) load_offsets(pos1);
             uint32_t D1 = 0u, vb1 = vb, rsel1 = rselw, lsel1 = lselw, U1 = 0u, rr = 0u, ll = 0u;
-            if (!ROW) {
+            auto next_pass = [&] {
+                ahead -= skip + len1;
+                if (PEEL) {
+                    bar_sync_if(ahead < 0 && taken < phases, 1 + grp, 64);
+                    taken -= ahead >> 31;
+                    ahead += (ahead >> 31) & Rg::kPhase;
+                } else if (ahead < 0) {
+                    if (taken < phases) bar_sync(1 + grp, 64);
+                    ++taken;
+                    ahead += Rg::kPhase;
+                }
+                if (POTTS) load_offsets(pos1);
+                if (ROW) return;
                 vb1 = valid_of(qi1);
                 R1 = spins(raw_load(y1, qi1), qi1, vb1);
                 D1 = spins(raw_load(y1 + 1 == L ? 0 : y1 + 1, qi1), qi1, vb1);
@@ -494,7 +511,9 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                 ll = spins(raw_load(y1, nl - 1), nl - 1, m);
                 rsel1 = rsel_of(qi1);
                 lsel1 = lsel_of(qi1);
-            }
+            };
+
+            if (!PEEL) next_pass();
 
             // ---- predict
             // (ROW) all ones in the lane of the row's last site if site 0 is changed: site 0's
@@ -514,9 +533,9 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                     }
                 }
             }
-            uint32_t dm, Rw, Q, e, k0, k1, da, SNr = 0u, SNl = 0u, nib = 0u;
+            uint32_t dm, lm, N, X, Q, e, Rw, k0, k1, da, SNr = 0u, SNl = 0u, RN1, LP1, T[4], df[4], bad, open, nib = 0u;
             int bin1, binw;
-            for (;;) {
+            auto attempt = [&](auto first_try) {
                 // the lane's four sites for either incoming bit (signs: 0 kept, 1 changed), then
                 // the incoming bits
                 uint32_t d0, d1, b0, b1;
@@ -542,9 +561,9 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                     d0 = sign_bytes(f0[0], f0[1], f0[2], f0[3]);
                     d1 = sign_bytes(f1[0], f1[1], f1[2], f1[3]);
                 }
-                // (the next pass's spins, neighbours and columns fill the gaps of this chain)
-                uint32_t RN1, LP1;
-                {
+                if constexpr (decltype(first_try)::value) {
+                    // (the next pass's spins, neighbours and columns fill the gaps of this chain)
+                    if (PEEL) next_pass();
                     if (POTTS) SN1 = (R1 + m + offn) & (7u * m);
                     RN1 = __shfl_sync(~0u, R1, rsrc & 31);
                     LP1 = __shfl_sync(~0u, R1, lsrc & 31);
@@ -572,7 +591,8 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                 const uint32_t cin = (uint32_t)((int)((b0 & prevbit) << prevshift) >> 31);
                 dm = select(cin, d1, d0) & vm;
                 // columns of the sites as they were met, bin changes plus EB
-                const uint32_t lm = __byte_perm(dm, cin, 0x2104), N = select(lm, n1, n0);
+                lm = __byte_perm(dm, cin, 0x2104);
+                N = select(lm, n1, n0);
                 e = select(dm, POTTS ? N : 4u * m - N, EB * m);
                 // sums over the lane's sites and the chain's lanes: bins before (X) and after (Q)
                 // every attempt are binw + byte
@@ -601,18 +621,17 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                 }
                 bin1 = bin + (int)tot - (int)(4u * EB * LPC);
                 binw = bin + (int)below - (int)lane_bias;
-                const uint32_t X = s * 256u + (POTTS ? 0x04080C10u : 0x02040608u);
+                X = s * 256u + (POTTS ? 0x04080C10u : 0x02040608u);
                 Q = s + (POTTS ? 0x0004080Cu : 0x00020406u);
                 const uint32_t rw = tab0 + ROWB * (uint32_t)binw;
                 // verify
-                uint32_t T[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     uint32_t ad = __dp4a(N, COLB << (8 * i), __dp4a(X, ROWB << (8 * i), rw));
                     T[i] = table_load<TAB>(tab_g, ad);
                 }
                 Rw = POTTS ? select(dm, SN, R) : R ^ (dm & m);
-                if (!POTTS) {
+                if (!POTTS && !PEEL) {
                     nib = pack4(Rw);
                     nib |= __shfl_down_sync(~0u, nib, 1) << 4;
                 }
@@ -622,11 +641,14 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                     columns(R1, SN1, D1, qi1 == nl - 1 ? (q == 0 ? fw : first) : RN1, lane == 0 && q1 > 0 ? pv : LP1, 0u,
                             SNl, rsel1, lsel1, k0, k1, da);
                 }
-                uint32_t df[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) df[i] = u[i] - T[i];
-                const uint32_t open = min(min(df[0], df[1]), min(df[2], df[3]));  // zero: a test is open
-                uint32_t bad = (sign_bytes(df[0], df[1], df[2], df[3]) ^ dm) & vm;
+                open = min(min(df[0], df[1]), min(df[2], df[3]));  // zero: a test is open
+                bad = (sign_bytes(df[0], df[1], df[2], df[3]) ^ dm) & vm;
+            };
+            if constexpr (PEEL) attempt(std::true_type{});
+            for (;;) {
+                if constexpr (!PEEL) attempt(std::true_type{});
                 if (!__any_sync(~0u, bad != 0u || open == 0u)) break;
                 if (__any_sync(~0u, open == 0u)) {
                     // draws that equal their entries: the 32-bit tests decide
@@ -662,6 +684,7 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                         B0 = l ? B0 : T[i];
                     }
                 }
+                if constexpr (PEEL) attempt(std::false_type{});
             }
 
             // ---- the next pass's candidates and draws (their latency is hidden by what follows)
@@ -672,6 +695,10 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                 dalt = ROW ? da : 0u;
                 load_candidates(tab0 + ROWB * (uint32_t)bin1);
                 load_draws(pos1);
+                if (!POTTS && PEEL) {
+                    nib = pack4(Rw);
+                    nib |= __shfl_down_sync(~0u, nib, 1) << 4;
+                }
             }
             // ---- commit
             {
