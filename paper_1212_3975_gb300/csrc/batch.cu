@@ -66,7 +66,7 @@ __device__ __forceinline__ SweepArgs batch_args(const BatchJob &j, int n_sweeps,
 template <int MODEL, int LPC, bool ROW, int TAB, int HMODE>
 __device__ __forceinline__ void body(const SweepArgs &a, const BatchJob &j, int cblk, uint32_t *smem)
 {
-    sweep_body<MODEL, LPC, ROW, true, TAB, HMODE, false>(a, cblk, kBatchGroups, j.lattice != 0, smem);
+    sweep_body<MODEL, LPC, ROW, true, TAB, HMODE, false, false>(a, cblk, kBatchGroups, j.lattice != 0, smem);
 }
 
 template <int MODEL, bool HIST>

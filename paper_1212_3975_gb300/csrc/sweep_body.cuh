@@ -195,7 +195,11 @@ struct StateCounts {
 // PEEL: the first attempt of a pass is code of its own, in whose gaps the next pass is
 // prepared, and a repetition does without that.  Shorter passes while latency bounds them,
 // more code than the instruction caches like where a scheduler has three deciding warps.
-template <int MODEL, int LPC, bool ROW, bool AL, int TAB, int HMODE, bool PEEL>
+// TWO: a row is two passes (128 < L <= 256): every lane keeps the spins of both in
+// registers (a pass's row below is the spins of the pass two on, its decisions the row
+// above of the pass two on), so that a pass reads four sites per lane of the lattice where
+// rows of any length read five quads (256 x 256, p = 8192, 4 sweeps: 7.6 ms against 8.8).
+template <int MODEL, int LPC, bool ROW, bool AL, int TAB, int HMODE, bool PEEL, bool TWO>
 __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, const int G, const bool stage_lattice,
                                            uint32_t *smem)
 {
@@ -210,6 +214,7 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
     constexpr bool HIST = HMODE != kHistNone;
     static_assert(ROW || LPC == 32, "long rows take whole warps");
     static_assert(ROW || !PEEL, "rows of one pass");
+    static_assert(!ROW || !TWO, "one pass or two");
     static_assert(AL || HMODE != kHistPairs, "pairs lie within a lane's four sites");
     __syncthreads();  // (persistent kernel: smem may still be read by the previous unit)
     const int tid = threadIdx.x, nt = block_threads(G), lane = tid & 31, warp = tid >> 5;
@@ -350,9 +355,12 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
         int y = 0, q = 0, qi = cl;  // (long rows) row, pass of the row; quad of the row
         uint32_t vb = valid_of(qi), vm = vb * 255u;
         // (ROW) this lane's spins of the rows being decided and three rows on: byte offsets
+        // (TWO: of the row two on; the second pass's share is own1 bytes further)
         uint8_t *const own = lat + (POTTS ? 4 * min(cl, nl - 1) : min(cl, nl - 1) >> 1);
         const uint32_t allb = rowb * (uint32_t)L;
-        uint32_t o0 = 0u, o3 = L > 3 ? 3u * rowb : 0u;
+        uint32_t o0 = 0u, o3 = TWO ? 2u * rowb : L > 3 ? 3u * rowb : 0u;
+        const uint32_t own1 = (uint32_t)(POTTS ? 4 * (min(LPC + cl, nl - 1) - cl) : (min(LPC + cl, nl - 1) >> 1) - (cl >> 1));
+        const uint32_t vb2 = valid_of(LPC + cl);  // (TWO) sites of the second pass
         // neighbouring quads: shuffle sources and byte selectors (a row's ends wrap)
         const int base = ch * LPC;
         const int rsrc = ROW ? base + (cl >= nl - 1 ? 0 : cl + 1) : lane + 1;
@@ -393,9 +401,16 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
         int bin = bin0;
         uint32_t R = spins(raw_load(0, qi), qi, vb), SN = 0u;
         uint32_t R1 = 0u, SN1 = 0u, raw2 = 0u;
+        uint32_t R2 = 0u, W1 = 0u;  // (TWO) the spins of the pass after the next, the new spins of the pass before
         if (ROW) {
             R1 = spins(raw_load(1, qi), qi, vb);
             raw2 = raw_load(2, qi);
+        }
+        if (TWO) {
+            R1 = spins(raw_load(0, LPC + cl), cl, vb2);
+            R2 = spins(raw_load(1, cl), cl, vb);
+            raw2 = raw_load(1, LPC + cl);
+            W1 = spins(raw_load(L - 1, LPC + cl), cl, vb2);
         }
 
         // columns of the pass's sites with the left neighbour kept (n0) / changed (n1); dalt:
@@ -479,9 +494,9 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
             int y1 = y, q1 = q + 1;
             if (!ROW && lastq) {
                 q1 = 0;
-                y1 = y + 1 == L ? 0 : y + 1;
+                if (!TWO) y1 = y + 1 == L ? 0 : y + 1;
             }
-            const bool last_row = ROW ? o0 + rowb == allb : y == L - 1;
+            const bool last_row = ROW || TWO ? o0 + rowb == allb : y == L - 1;
             const int qi1 = ROW ? cl : q1 * LPC + cl;
             // its draws
             const int len = ROW ? L : min(4 * LPC, L - 4 * LPC * q), len1 = ROW ? L : min(4 * LPC, L - 4 * LPC * q1);
@@ -502,6 +517,14 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                 }
                 if (POTTS) load_offsets(pos1);
                 if (ROW) return;
+                if (TWO) {
+                    vb1 = q1 ? vb2 : active ? m : 0u;
+                    D1 = spins(raw2, cl, vb1);
+                    U1 = W1;
+                    rsel1 = rsel_of(qi1);
+                    lsel1 = lsel_of(qi1);
+                    return;
+                }
                 vb1 = valid_of(qi1);
                 R1 = spins(raw_load(y1, qi1), qi1, vb1);
                 D1 = spins(raw_load(y1 + 1 == L ? 0 : y1 + 1, qi1), qi1, vb1);
@@ -565,7 +588,9 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                     // (the next pass's spins, neighbours and columns fill the gaps of this chain)
                     if (PEEL) next_pass();
                     if (POTTS) SN1 = (R1 + m + offn) & (7u * m);
-                    RN1 = __shfl_sync(~0u, R1, rsrc & 31);
+                    // (TWO, first pass: to lane 31's right is the second pass, to lane 0's left its
+                    // last quad)
+                    RN1 = __shfl_sync(~0u, TWO && lane == 0 && q1 == 0 ? R2 : R1, rsrc & 31);
                     LP1 = __shfl_sync(~0u, R1, lsrc & 31);
                     if (POTTS) {
                         SNl = __shfl_sync(~0u, SN1, lsrc & 31);
@@ -575,7 +600,8 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                         D1 = spins(raw2, cl, vb);
                         columns(R1, SN1, D1, RN1, LP1, SNr, SNl, rsel1, lsel1, k0, k1, da);
                     } else {
-                        RN1 = lane == 31 ? rr : RN1;
+                        if (TWO) ll = __shfl_sync(~0u, R2, nl - 1 - LPC);
+                        else RN1 = lane == 31 ? rr : RN1;
                         LP1 = lane == 0 && q1 == 0 ? ll : LP1;
                     }
                 }
@@ -638,7 +664,7 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                 if (!ROW) {
                     // the row's first quad, and the quad before the next pass
                     const uint32_t fw = __shfl_sync(~0u, Rw, 0), pv = __shfl_sync(~0u, Rw, 31);
-                    columns(R1, SN1, D1, qi1 == nl - 1 ? (q == 0 ? fw : first) : RN1, lane == 0 && q1 > 0 ? pv : LP1, 0u,
+                    columns(R1, SN1, D1, qi1 == nl - 1 ? (TWO || q == 0 ? fw : first) : RN1, lane == 0 && q1 > 0 ? pv : LP1, 0u,
                             SNl, rsel1, lsel1, k0, k1, da);
                 }
 #pragma unroll
@@ -702,7 +728,7 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
             }
             // ---- commit
             {
-                uint8_t *const r = ROW ? own + o0 : lat + (size_t)y * rowb + (POTTS ? 4 * qi : qi >> 1);
+                uint8_t *const r = ROW ? own + o0 : TWO ? own + (o0 + (q ? own1 : 0u)) : lat + (size_t)y * rowb + (POTTS ? 4 * qi : qi >> 1);
                 if (POTTS) {
                     if (vb) *reinterpret_cast<volatile uint32_t *>(r) = Rw;
                 } else {
@@ -710,7 +736,7 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                 }
             }
             __syncwarp();  // other lanes read these spins
-            if (!ROW && q == 0) first = __shfl_sync(~0u, Rw, 0);
+            if (!ROW && !TWO && q == 0) first = __shfl_sync(~0u, Rw, 0);
             if (HIST) {
                 constexpr bool part = !AL;  // (a row's last lane has fewer than four sites)
                 if (HMODE == kHistPairs) {
@@ -815,6 +841,19 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                              : (uint32_t) * reinterpret_cast<const volatile uint8_t *>(own + o3);
                 o0 = last_row ? 0u : o0 + rowb;
                 o3 = o3 + rowb == allb ? 0u : o3 + rowb;
+            }
+            if (TWO) {
+                R1 = R2;
+                R2 = D1;
+                W1 = Rw;
+                // (final by now: the row below the pass after next)
+                const uint8_t *const r = own + (o3 + (q ? own1 : 0u));
+                raw2 = POTTS ? *reinterpret_cast<const volatile uint32_t *>(r)
+                             : (uint32_t) * reinterpret_cast<const volatile uint8_t *>(r);
+                if (lastq) {
+                    o0 = last_row ? 0u : o0 + rowb;
+                    o3 = o3 + rowb == allb ? 0u : o3 + rowb;
+                }
             }
             if (!ROW) {
                 vb = vb1;

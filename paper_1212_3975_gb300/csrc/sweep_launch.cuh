@@ -12,17 +12,17 @@ namespace sweep {
 // passes repeat often (64 x 64, p = 1024): 4.13 / 4.24 ms.
 constexpr int kPeelGroups = 6;
 
-template <int MODEL, int LPC, bool ROW, bool AL, int TAB, int HMODE, bool PEEL>
+template <int MODEL, int LPC, bool ROW, bool AL, int TAB, int HMODE, bool PEEL, bool TWO>
 __global__ void __launch_bounds__(block_threads(kMaxGroups), 1) sweep_kernel(SweepArgs a, int groups, bool stage_lattice)
 {
     extern __shared__ __align__(16) uint32_t smem[];
-    sweep_body<MODEL, LPC, ROW, AL, TAB, HMODE, PEEL>(a, blockIdx.x, groups, stage_lattice, smem);
+    sweep_body<MODEL, LPC, ROW, AL, TAB, HMODE, PEEL, TWO>(a, blockIdx.x, groups, stage_lattice, smem);
 }
 
-template <int MODEL, int LPC, bool ROW, bool AL, int TAB, int HMODE, bool PEEL>
+template <int MODEL, int LPC, bool ROW, bool AL, int TAB, int HMODE, bool PEEL, bool TWO>
 cudaError_t launch_as(const SweepLaunch &l)
 {
-    auto kern = sweep_kernel<MODEL, LPC, ROW, AL, TAB, HMODE, PEEL>;
+    auto kern = sweep_kernel<MODEL, LPC, ROW, AL, TAB, HMODE, PEEL, TWO>;
     if (l.shape.smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.shape.smem);
         if (e != cudaSuccess) return e;
@@ -35,8 +35,10 @@ template <int MODEL, int LPC, bool ROW, bool AL, int TAB, int HMODE>
 cudaError_t launch(const SweepLaunch &l)
 {
     if constexpr (ROW && TAB != kTabShared16)
-        if (l.shape.groups <= kPeelGroups) return launch_as<MODEL, LPC, ROW, AL, TAB, HMODE, true>(l);
-    return launch_as<MODEL, LPC, ROW, AL, TAB, HMODE, false>(l);
+        if (l.shape.groups <= kPeelGroups) return launch_as<MODEL, LPC, ROW, AL, TAB, HMODE, true, false>(l);
+    if constexpr (!ROW)
+        if (l.args.L <= 8 * LPC) return launch_as<MODEL, LPC, ROW, AL, TAB, HMODE, false, true>(l);
+    return launch_as<MODEL, LPC, ROW, AL, TAB, HMODE, false, false>(l);
 }
 
 template <int L, bool HIST>
