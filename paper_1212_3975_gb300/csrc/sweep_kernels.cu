@@ -137,12 +137,15 @@ int hist_mode(const SweepPlan &pl)
                                                                                            : sweep::kHistSingle;
 }
 
-// Groups per block (`groups` > 0: that many).  A pass takes some 700 cycles with one
-// deciding warp per scheduler and then 60 more per group of the SM (64 x 64: 670 cycles in
-// blocks of 4 groups, 845 of 6, 930 of 8, 1110 of 12); blocks beyond one per SM wait for
-// another wave.  (At 170 cycles per group more waves of smaller blocks were taken:
-// 256 x 256, p = 8192, 6 waves of 9 groups 7.62 ms, 5 of 11 6.83 ms; 64 x 64, p = 16000,
-// 10 sweeps, 6 of 9 2.14 ms, 5 of 11 1.95 ms.)
+// Groups per block (`groups` > 0: that many).  A pass takes some 680 cycles with one
+// deciding warp per scheduler, and 600 and 42 more per group with two or three (64 x 64:
+// 670 cycles in blocks of 4 groups, 845 of 6, 930 of 8, 1110 of 12); blocks beyond one per
+// SM wait for another wave.  (At 170 cycles per group more waves of smaller blocks were
+// taken: 256 x 256, p = 8192, 6 waves of 9 groups 7.62 ms, 5 of 11 6.83 ms; 64 x 64,
+// p = 16000, 10 sweeps, 6 of 9 2.14 ms, 5 of 11 1.95 ms.)  Of equal costs the fewest
+// groups, on more SMs, deciding and drawing warps on schedulers of their own (8-Potts
+// 32 x 32, p = 639, 2 or 1 groups instead of 4: 413 against 530 us; 8 x 8, p = 1024:
+// 291 against 352).
 SweepShape sweep_shape(const muca_ctx *ctx, const SweepPlan &pl, bool hist, int groups)
 {
     SweepShape s;
@@ -160,8 +163,8 @@ SweepShape sweep_shape(const muca_ctx *ctx, const SweepPlan &pl, bool hist, int 
         for (int n = 1; n <= std::min<long>(sweep::kMaxGroups, all); ++n) {
             if (n > 1 && launch_smem(ctx, pl, hist, staged(n), n, s.lpc) > (size_t)kMaxSmem) break;
             const long waves = ((all + n - 1) / n + ctx->n_sm - 1) / ctx->n_sm;
-            const double t = (double)waves * std::max(700.0, 400.0 + 60.0 * n);
-            if (best == 0.0 || t <= best) {
+            const double t = (double)waves * (n <= 4 ? 680.0 : 600.0 + 42.0 * n);
+            if (best == 0.0 || t < best) {
                 best = t;
                 G = n;
             }

@@ -23,8 +23,8 @@ template <int MODEL, int LPC, bool ROW, bool AL, int TAB, int HMODE, bool PEEL, 
 cudaError_t launch_as(const SweepLaunch &l)
 {
     auto kern = sweep_kernel<MODEL, LPC, ROW, AL, TAB, HMODE, PEEL, TWO>;
-    if (l.shape.smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.shape.smem);
+    if (l.shape.smem > 48 * 1024) {  // (one limit for all: another thread may launch the kernel too)
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
         if (e != cudaSuccess) return e;
     }
     kern<<<l.blocks, block_threads(l.shape.groups), l.shape.smem, l.stream>>>(l.args, l.shape.groups, l.shape.lattice);
@@ -53,7 +53,7 @@ cudaError_t launch_small_as(const SweepLaunch &l)
 {
     auto kern = small_kernel<L, HIST>;
     if (l.shape.smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.shape.smem);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
         if (e != cudaSuccess) return e;
     }
     kern<<<l.blocks, block_threads(l.shape.groups), l.shape.smem, l.stream>>>(l.args, l.shape.groups);
