@@ -85,6 +85,9 @@ __device__ __forceinline__ void run_unit(const SweepArgs &a, const BatchJob &j, 
             }
         }
         break;
+    case 2:
+        if constexpr (MODEL == MUCA_POTTS) body<MODEL, 2, true, kTabShared, HP>(a, j, cblk, smem);
+        break;
     case 4:
         if constexpr (MODEL == MUCA_POTTS) body<MODEL, 4, true, kTabShared, HP>(a, j, cblk, smem);
         break;

@@ -69,7 +69,7 @@ struct Ring {
     static constexpr int kStride = kSites + 4 * LPC, kByteStride = kStride + 8;
 };
 // shared memory of a group: its ring, and a byte per lane for the sums over lanes
-__host__ __device__ constexpr size_t ring_bytes(int model) { return 6656 + (model == MUCA_POTTS ? 1664 + 8 * 8 : 0) + 32; }
+__host__ __device__ constexpr size_t ring_bytes(int model) { return 6656 + (model == MUCA_POTTS ? 1664 + 8 * 16 : 0) + 32; }
 
 __device__ __forceinline__ void bar_sync(int id, int n)
 {
@@ -324,16 +324,17 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
         const uint32_t offs_s = (uint32_t)__cvta_generic_to_shared(offs_of(grp));
         const uint32_t hist_s = (uint32_t)__cvta_generic_to_shared(s_hist);
         const uint32_t dummy = hist_s + 4u * (uint32_t)(((n_hist + 3) & ~3) + lane);
-        const uint32_t starts = LPC == 4 ? 0x11111111u : LPC == 8 ? 0x01010101u : LPC == 16 ? 0x00010001u : 1u;
+        const uint32_t starts = LPC == 2 ? 0x55555555u : LPC == 4 ? 0x11111111u : LPC == 8 ? 0x01010101u : LPC == 16 ? 0x00010001u : 1u;
         const uint32_t prevbit = cl == 0 ? 0u : 1u << (lane - 1);
         const int prevshift = (32 - lane) & 31;  // ... to bit 31
         // sums over the lanes of a chain: each lane's as a byte in shared memory, read back as
         // words and summed up to the lane by byte products (a shuffle scan takes twice as long)
         const uint32_t sums_s = (uint32_t)__cvta_generic_to_shared(s_ring) +
                                 (uint32_t)((grp + 1) * (int)ring_bytes(MODEL) - 32 + LPC * ch);
-        uint32_t lower[LPC / 4];  // 1 in the bytes of the lanes below this one
+        constexpr int NW = LPC < 4 ? 1 : LPC / 4;  // words of the lanes' bytes
+        uint32_t lower[NW];  // 1 in the bytes of the lanes below this one
 #pragma unroll
-        for (int k = 0; k < LPC / 4; ++k)
+        for (int k = 0; k < NW; ++k)
             lower[k] = cl >= 4 * k + 4 ? m : cl <= 4 * k ? 0u : m & ((1u << (8 * (cl - 4 * k))) - 1u);
         const uint32_t lane_bias = BB + 4u * EB * (uint32_t)cl;
 
@@ -627,8 +628,12 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                 {
                     asm volatile("st.shared.u8 [%0], %1;" ::"r"(sums_s + (uint32_t)cl), "r"(s >> 24) : "memory");
                     __syncwarp();
-                    uint32_t w[LPC / 4];
-                    if constexpr (LPC == 4) {
+                    uint32_t w[NW];
+                    if constexpr (LPC == 2) {
+                        uint16_t h;
+                        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(h) : "r"(sums_s) : "memory");
+                        w[0] = h;
+                    } else if constexpr (LPC == 4) {
                         asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w[0]) : "r"(sums_s) : "memory");
                     } else if constexpr (LPC == 8) {
                         asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(w[0]), "=r"(w[1]) : "r"(sums_s) : "memory");
@@ -641,9 +646,9 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                                          : "memory");
                     }
 #pragma unroll
-                    for (int k = 0; k < LPC / 4; ++k) below = __dp4a(w[k], lower[k], below);
+                    for (int k = 0; k < NW; ++k) below = __dp4a(w[k], lower[k], below);
 #pragma unroll
-                    for (int k = 0; k < LPC / 4; ++k) tot = __dp4a(w[k], m, tot);
+                    for (int k = 0; k < NW; ++k) tot = __dp4a(w[k], m, tot);
                 }
                 bin1 = bin + (int)tot - (int)(4u * EB * LPC);
                 binw = bin + (int)below - (int)lane_bias;

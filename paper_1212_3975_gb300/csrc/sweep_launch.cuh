@@ -105,6 +105,9 @@ cudaError_t launch_shape(const SweepLaunch &l, bool hist)
     case 1:
         if constexpr (MODEL == MUCA_ISING) return hist ? launch_small<true>(l) : launch_small<false>(l);
         return cudaErrorInvalidConfiguration;
+    case 2:
+        if constexpr (MODEL == MUCA_POTTS) return ts ? launch_hist<MODEL, 2, true, AL, kTabShared>(l, hist) : cudaErrorInvalidConfiguration;
+        return cudaErrorInvalidConfiguration;
     case 4:
         if constexpr (MODEL == MUCA_POTTS) return ts ? launch_hist<MODEL, 4, true, AL, kTabShared>(l, hist) : cudaErrorInvalidConfiguration;
         return cudaErrorInvalidConfiguration;
