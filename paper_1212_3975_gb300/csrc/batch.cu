@@ -22,9 +22,6 @@ namespace muca {
 namespace {
 using namespace sweep;
 
-// groups of chains per work unit (and 2 warps each per block)
-constexpr int kBatchGroups = 4;
-
 struct BatchUnit {
     int job, cblk;
 };
@@ -203,6 +200,13 @@ struct TuneChoice {
 };
 
 }  // namespace
+
+int batch_max_sweeps(const muca_ctx *ctx)
+{
+    const SweepShape shape = sweep_shape(ctx, plan_sweeps(ctx, false, kBatchGroups), true, kBatchGroups);
+    return max_launch_sweeps(shape.chains, ctx->V);
+}
+
 }  // namespace muca
 
 using namespace muca;
@@ -226,6 +230,7 @@ struct muca_batch {
     uint32_t *d_therm = nullptr;  // [n_jobs]: thermalisation sweep counters
     size_t smem = 0;
     int grid = 0, staging = MUCA_STAGING_AUTO, split = 1;
+    int max_sweeps = 1;  // sweeps per launch at most (the smallest limit of the jobs)
     int max_bins = 0, max_thr = 0, max_ktab = 0;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
@@ -257,6 +262,7 @@ int configure(muca_batch *b)
     b->h_jobs.assign(b->n_jobs, BatchJob{});
     b->plan_flags.assign(b->n_jobs, 0);
     b->smem = 0;
+    b->max_sweeps = 1 << 30;
     b->max_bins = b->max_thr = b->max_ktab = 0;
     std::vector<std::pair<long long, BatchUnit>> units;
     for (int i = 0; i < b->n_jobs; ++i) {
@@ -310,6 +316,7 @@ int configure(muca_batch *b)
         j.row = shape.row;
         b->plan_flags[i] = plan_flags(pl);
         b->smem = std::max(b->smem, shape.smem);
+        b->max_sweeps = std::min(b->max_sweeps, batch_max_sweeps(c));
         b->max_bins = std::max(b->max_bins, c->n_bins);
         b->max_thr = std::max(b->max_thr, c->n_bins * c->n_de);
         b->max_ktab = std::max(b->max_ktab, c->n_bins * ktab_width(c->model));
@@ -350,7 +357,7 @@ int configure(muca_batch *b)
 // Queue one weight iteration of every lattice on the batch stream.
 int enqueue_iteration(muca_batch *b, int n_sweeps)
 {
-    const int split = std::max(1, std::min(b->split, n_sweeps));
+    const int split = sweep_launches(n_sweeps, b->split, b->max_sweeps);
     for (int s = 0; s < split; ++s) {
         const int s0 = (int)((long long)n_sweeps * s / split), s1 = (int)((long long)n_sweeps * (s + 1) / split);
         if (s == 0) {
@@ -534,19 +541,10 @@ int muca_batch_plan(const muca_batch *b, int j)
 }
 
 namespace {
-// Before a call that queues iterations: sweep launches per iteration, pending tables
-// of individual contexts, and the iteration counters of the random streams.
-int begin_iterations(muca_batch *b, int n_sweeps)
+// Before a call that queues iterations: pending threshold tables of individual contexts,
+// and the iteration and thermalisation counters of the random streams.
+int begin_iterations(muca_batch *b)
 {
-    // uint32 block histograms: at most 32 chains x sweeps x sites per launch below 2^31
-    long long vmax = 0;
-    for (muca_ctx *c : b->ctx) vmax = std::max<long long>(vmax, c->V);
-    while (32LL * ((n_sweeps + b->split - 1) / b->split) * vmax >= (1LL << 31)) {
-        b->split *= 2;
-        drop_graph(b);
-    }
-    // pending threshold tables of individual contexts, iteration and thermalisation
-    // counters
     std::vector<uint32_t> it(b->n_jobs), th(b->n_jobs);
     for (int i = 0; i < b->n_jobs; ++i) {
         muca_ctx *c = b->ctx[i];
@@ -571,7 +569,7 @@ int muca_batch_iterate(muca_batch *b, int n_iterations, int n_sweeps, int use_gr
     MUCA_RANGE("muca_batch_iterate");
     if (!b) return fail(MUCA_ERR_ARG, "null batch");
     if (n_iterations < 1 || n_sweeps < 1) return fail(MUCA_ERR_ARG, "need n_iterations >= 1 and n_sweeps >= 1");
-    int rc0 = begin_iterations(b, n_sweeps);
+    int rc0 = begin_iterations(b);
     if (rc0) return rc0;
     if (use_graph) {
         if (!b->gexec || b->g_iters != n_iterations || b->g_sweeps != n_sweeps) {
@@ -595,7 +593,7 @@ int muca_batch_iterate(muca_batch *b, int n_iterations, int n_sweeps, int use_gr
             b->g_sweeps = n_sweeps;
         }
         MUCA_CUDA_TRY(cudaGraphLaunch(b->gexec, b->stream));
-        note_launches((uint64_t)n_iterations * (5 + b->split));
+        note_launches((uint64_t)n_iterations * (5 + sweep_launches(n_sweeps, b->split, b->max_sweeps)));
     } else {
         for (int i = 0; i < n_iterations; ++i) {
             int rc = enqueue_iteration(b, n_sweeps);
@@ -638,7 +636,7 @@ int muca_batch_converge(muca_batch *b, int n_sweeps, int therm_sweeps, int max_i
     if (!b) return fail(MUCA_ERR_ARG, "null batch");
     if (n_sweeps < 1 || max_iterations < 1 || therm_sweeps < 0)
         return fail(MUCA_ERR_ARG, "need n_sweeps >= 1, therm_sweeps >= 0 and max_iterations >= 1");
-    int rc = begin_iterations(b, n_sweeps);
+    int rc = begin_iterations(b);
     if (rc) return rc;
     const int nb = (b->n_jobs + 255) / 256;
     batch_fill_kernel<<<nb, 256, 0, b->stream>>>(b->d_active, b->n_jobs, 1);

@@ -118,6 +118,23 @@ struct SweepShape {
     size_t smem;
 };
 
+// Sweeps of one launch at most, `chains` chains per block: a block's 32-bit histogram
+// counts (every chain in one bin), the sums of them that its flush makes and the draw
+// positions stay below 2^31.
+inline int max_launch_sweeps(int chains, int V)
+{
+    const uint64_t per_sweep = (uint64_t)(chains > 32 ? chains : 32) * (uint64_t)(V + 3), n = (1ull << 31) / per_sweep;
+    return n < 1 ? 1 : n > (1u << 30) ? 1 << 30 : (int)n;
+}
+// Launches that n_sweeps sweeps take: `split` or as many as `most` sweeps per launch need
+// (launch s of them makes the sweeps from n s / launches to n (s + 1) / launches).
+inline int sweep_launches(int n_sweeps, int split, int most)
+{
+    const int need = n_sweeps / most + (n_sweeps % most != 0);
+    const int n = split > need ? split : need;
+    return n < 1 ? 1 : n < n_sweeps ? n : n_sweeps;
+}
+
 // Device view of one lattice of a batch (pointers into its context).
 struct BatchJob {
     int model, L, q, p, p_pad, row_words, lat_words, n_bins, n_de, V;
@@ -232,6 +249,9 @@ SweepPlan plan_sweeps(const muca_ctx *ctx, bool allow_compact = true, int groups
 SweepShape sweep_shape(const muca_ctx *ctx, const SweepPlan &pl, bool hist, int groups = 0);
 int hist_mode(const SweepPlan &pl);
 int plan_flags(const SweepPlan &pl);  // MUCA_PLAN_* bit mask
+constexpr int kBatchGroups = 4;       // groups of chains per work unit of a batch
+// sweeps of one launch of a batch that holds this lattice, at most
+int batch_max_sweeps(const muca_ctx *ctx);
 cudaError_t launch_batch_update(const BatchJob *d_jobs, int n_jobs, int max_bins, int max_thr, cudaStream_t st);
 int launch_ktab(muca_ctx *ctx);
 // kernel table: Ising [n_bins][5] by unequal neighbours, Potts [n_bins][9] by dE + 4

@@ -266,7 +266,8 @@ __device__ __forceinline__ void small_body(const SweepArgs &a, const int cblk, c
         if (c0 + c < a.p) a.lat[(size_t)c0 * lat_words + i] = s_lat[k * lw + c];
     }
     if (HIST) {
-        // a warp per bin: counts of the block's chains (padding chains left out)
+        // a warp per bin: counts of the block's chains (padding chains left out); all of a
+        // launch's are below 2^31 (max_launch_sweeps)
         for (int b = warp; b < n_bins; b += nt >> 5) {
             uint32_t x = 0u;
             for (int g = 0; g < G; ++g)

@@ -1,0 +1,65 @@
+"""Sizes of sweep launches, checked on the host over every lattice: 32-bit counts of a
+block stay below 2^31 whatever a batch is asked to do."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ISING, POTTS = 0, 1
+SIDES = [(ISING, L) for L in range(4, 1025, 2)] + [(POTTS, L) for L in range(3, 256)]
+
+
+@pytest.fixture(scope="module")
+def probe(tmp_path_factory):
+    from paper_1212_3975_gb300 import build as b
+    lib = b.build()
+    out = str(tmp_path_factory.mktemp("plan") / "plan_probe.so")
+    subprocess.run([b.nvcc(), *b.ARCH, *b.COMMON, "-shared", "-o", out, os.path.join(HERE, "plan_probe.cu"), lib,
+                    "-Xlinker", "-rpath=" + os.path.dirname(lib)], check=True)
+    return ctypes.CDLL(out)
+
+
+@pytest.fixture(scope="module")
+def muca():
+    import paper_1212_3975_gb300 as m
+    from paper_1212_3975_gb300 import build
+    build.build()
+    return m
+
+
+def test_batch_launches_keep_counts_in_32_bits(probe):
+    """Every attempt of a work unit of a batch may end in one bin.  (Draw positions and
+    passes are counted in 32 bits with sign.)"""
+    two = (ctypes.c_int * 2)()
+    for model, L in SIDES:
+        if L % 4:
+            continue
+        probe.probe_batch(model, L, 4096, two)
+        chains, most = two
+        assert chains * L * L * most < 2 ** 31 or most == 1, (model, L)
+        for n in (1, 7, most - 1, most, most + 1, 3 * most + 5, 2 ** 31 - 1):
+            for split in (1, 2, 64):
+                if not 0 < n < 2 ** 31:
+                    continue
+                k = probe.probe_launches(n, split, most)
+                assert 1 <= k <= n and k >= min(split, n)
+                assert max(n * (s + 1) // k - n * s // k for s in (0, k // 2, k - 1)) <= most, (model, L, n, split)
+
+
+@pytest.mark.gpu
+def test_batch_counts_all_attempts_of_a_cold_lattice(muca):
+    """128 chains of a 4 x 4 lattice that stay in the ground state: more than 2^32 counts of
+    one bin by one work unit, in one iteration."""
+    n, p = 4194303, 128
+    with muca.Muca(ISING, 4, 2, 1, 1) as g:
+        nb = g.n_bins
+    b = muca.MucaBatch([(ISING, 4, 2, p, 9)])
+    b.job(0).set_lnw(-3.0 * (4.0 * np.arange(nb) - 32.0))
+    b.iterate(1, n)
+    H = b.job(0).get_histogram()
+    b.close()
+    assert int(H.sum()) == n * p * 16
+    assert int(H.max()) > 2 ** 32
