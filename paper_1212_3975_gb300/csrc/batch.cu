@@ -610,11 +610,11 @@ int muca_batch_iterate(muca_batch *b, int n_iterations, int n_sweeps, int use_gr
 }
 
 namespace {
-// Thermalisation sweeps of every running lattice (no histogram), in launches that
-// keep the uint32 block histogram bound of the iteration launches.
+// Thermalisation sweeps of every running lattice (no histogram), in launches of at most
+// b->max_sweeps: the bodies count their draws in 32 bits.
 int enqueue_thermalization(muca_batch *b, int n_sweeps)
 {
-    const int split = std::max(1, std::min(b->split, n_sweeps));
+    const int split = sweep_launches(n_sweeps, b->split, b->max_sweeps);
     for (int s = 0; s < split; ++s) {
         const int s0 = (int)((long long)n_sweeps * s / split), s1 = (int)((long long)n_sweeps * (s + 1) / split);
         MUCA_CUDA_TRY(cudaMemsetAsync(b->d_queue, 0, sizeof(unsigned), b->stream));

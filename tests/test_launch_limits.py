@@ -63,3 +63,26 @@ def test_batch_counts_all_attempts_of_a_cold_lattice(muca):
     b.close()
     assert int(H.sum()) == n * p * 16
     assert int(H.max()) > 2 ** 32
+
+
+@pytest.mark.gpu
+def test_batch_thermalisation_beyond_one_launch(muca):
+    """Intermediate thermalisation is cut into launches by its own length (the iterations
+    around it are short), and continues like a single context's."""
+    job = (ISING, 4, 2, 40, 3)
+
+    def run(therm):
+        b = muca.MucaBatch([job])
+        before = muca.kernel_launches()
+        b.converge(5, 2, therm_sweeps=therm)
+        launches = muca.kernel_launches() - before
+        spins, lnw = b.job(0).get_spins(), b.job(0).get_lnw()
+        b.close()
+        return launches, spins, lnw
+
+    few = run(10)[0]
+    launches, spins, lnw = run(900000)   # 128 chains x 16 sites x 900000 sweeps: two launches
+    assert launches == few + 1
+    with muca.Muca(*job) as g:
+        g.converge(5, 2, therm_sweeps=900000)
+        assert np.array_equal(g.get_spins(), spins) and np.array_equal(g.get_lnw(), lnw)
