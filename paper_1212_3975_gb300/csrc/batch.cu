@@ -270,13 +270,13 @@ int configure(muca_batch *b)
         c->cfg.staging = b->staging;
         if (c->cfg.ensemble != MUCA_ENSEMBLE_ENERGY)
             return fail(MUCA_ERR_ARG, "batched lattices need the energy ensemble (job " + std::to_string(i) + ")");
+        if (c->L % 4 != 0)
+            return fail(MUCA_ERR_ARG, "batched lattices need L % 4 == 0 (job " + std::to_string(i) + ")");
         const SweepPlan pl = plan_sweeps(c, false, kBatchGroups);
         const SweepShape shape = sweep_shape(c, pl, true, kBatchGroups);
         // (pairs wherever the table is in shared memory: run_unit)
         if (shape.groups != kBatchGroups || (shape.lpc > 1 && pl.hist_pairs != pl.table_smem))
             return fail(MUCA_ERR_ARG, "batched staging exceeds shared memory");
-        if (c->L % 4 != 0)
-            return fail(MUCA_ERR_ARG, "batched lattices need L % 4 == 0 (job " + std::to_string(i) + ")");
         BatchJob &j = b->h_jobs[i];
         j.model = c->model;
         j.L = c->L;
