@@ -344,11 +344,16 @@ int configure(muca_batch *b)
     MUCA_CUDA_TRY(cudaMemcpyAsync(b->d_jobs, b->h_jobs.data(), sizeof(BatchJob) * b->n_jobs, cudaMemcpyHostToDevice,
                                   b->stream));
     MUCA_CUDA_TRY(cudaStreamSynchronize(b->stream));
-    if (b->smem > 227 * 1024) return fail(MUCA_ERR_ARG, "batched staging exceeds shared memory");
-    MUCA_CUDA_TRY(
-        cudaFuncSetAttribute(batch_sweep_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem));
-    MUCA_CUDA_TRY(
-        cudaFuncSetAttribute(batch_sweep_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem));
+    // one limit for all batches, which share the two kernels (a limit of each batch's own
+    // size would take away from a larger one that is there already): what the kernels' own
+    // variables leave of a block's shared memory
+    for (const void *kern : {(const void *)batch_sweep_kernel<false>, (const void *)batch_sweep_kernel<true>}) {
+        cudaFuncAttributes at;
+        MUCA_CUDA_TRY(cudaFuncGetAttributes(&at, kern));
+        const size_t most = (size_t)kMaxSmem - at.sharedSizeBytes;
+        if (b->smem > most) return fail(MUCA_ERR_ARG, "batched staging exceeds shared memory");
+        MUCA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
+    }
     if (b->grid <= 0) b->grid = std::min(b->n_units, sm_count());
     drop_graph(b);
     return MUCA_OK;

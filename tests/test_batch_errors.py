@@ -1,4 +1,4 @@
-"""What a batch refuses, and with which reason."""
+"""What a batch refuses, and with which reason; batches beside each other."""
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -21,3 +21,14 @@ def test_ragged_side_names_the_reason(muca, job):
         muca.MucaBatch([(ISING, 8, 2, 8, 1), job])
     assert ei.value.code == muca._muca.MUCA_ERR_ARG
     assert "L % 4 == 0 (job 1)" in str(ei.value)
+
+
+def test_a_smaller_batch_leaves_a_larger_one_its_shared_memory(muca):
+    large = muca.MucaBatch([(ISING, 64, 2, 8, 1)])
+    small = muca.MucaBatch([(ISING, 8, 2, 8, 1)])
+    large.iterate(1, 2)
+    small.iterate(1, 2)
+    assert int(large.job(0).get_histogram().sum()) == 2 * 8 * 64 * 64
+    assert int(small.job(0).get_histogram().sum()) == 2 * 8 * 8 * 8
+    small.close()
+    large.close()
