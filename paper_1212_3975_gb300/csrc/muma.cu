@@ -45,6 +45,13 @@ struct MumaArgs {
     uint32_t sweep0, iteration, ctr3, key0;
 };
 
+// One thread per chain, one lattice word at a time: the word being decided and the words
+// above and below it stay in registers, so a site reads nothing of the lattice.  With five
+// bit loads per site the lanes of a warp, whose lattices lie L x row_words words apart, cost
+// up to 32 cache lines per load.  Time of a chain's attempt at p = 4096 with bit loads, with
+// bit loads of lattices interleaved word by word, and with words in registers: 64 x 64 557,
+// 348 and 205 ns; 32 x 32 508, 284 and 171; 8 x 8 297, 275 and 172.  Bound by the chain's
+// serial step: the table load that depends on M, the test, and a quarter of a Philox block.
 template <bool HIST, bool SMEM_HIST>
 __global__ void __launch_bounds__(128) muma_sweep_kernel(MumaArgs a)
 {
@@ -57,32 +64,47 @@ __global__ void __launch_bounds__(128) muma_sweep_kernel(MumaArgs a)
     if (c < a.p) {
         const int L = a.L, V = L * L, RW = a.row_words;
         uint32_t *lat = a.lat + (size_t)c * (size_t)(L * RW);
-        auto bit = [&](int x, int y) -> uint32_t { return (lat[y * RW + (x >> 5)] >> (x & 31)) & 1u; };
         int E = a.E[c], M = a.M[c];
         for (int sw = 0; sw < a.n_sweeps; ++sw) {
             const uint32_t sweep = a.sweep0 + (uint32_t)sw;
             uint4 blk = make_uint4(0u, 0u, 0u, 0u);
-            for (int i = 0; i < V; ++i) {
-                if ((i & 3) == 0 || i == 0)
-                    blk = philox4x32_10(make_uint4((uint32_t)i >> 2, sweep, a.iteration, a.ctr3), a.key0, (uint32_t)c);
-                const uint32_t u = (i & 3) == 0 ? blk.x : (i & 3) == 1 ? blk.y : (i & 3) == 2 ? blk.z : blk.w;
-                const int x = i % L, y = i / L;
-                const uint32_t me = bit(x, y);
-                const int unequal = (int)((bit(x == L - 1 ? 0 : x + 1, y) ^ me) + (bit(x == 0 ? L - 1 : x - 1, y) ^ me) +
-                                          (bit(x, y == L - 1 ? 0 : y + 1) ^ me) + (bit(x, y == 0 ? L - 1 : y - 1) ^ me));
-                const int b = (M + V) >> 1;
-                const uint32_t A = a.thr[b * 10 + (me ? 5 : 0) + unequal];
-                if (A == kAlways || u < A) {
-                    lat[y * RW + (x >> 5)] ^= 1u << (x & 31);
-                    E += 8 - 4 * unequal;
-                    M -= me ? 2 : -2;
-                }
-                if (HIST) {
-                    const int bn = (M + V) >> 1;
-                    if (SMEM_HIST)
-                        atomicAdd(&s_hist[bn], 1u);
-                    else
-                        atomicAdd(reinterpret_cast<unsigned long long *>(&a.H[bn]), 1ull);
+            int i = 0;  // site
+            for (int y = 0; y < L; ++y) {
+                uint32_t *const row = lat + y * RW;
+                const uint32_t *const up = lat + (y == 0 ? L - 1 : y - 1) * RW;
+                const uint32_t *const down = lat + (y == L - 1 ? 0 : y + 1) * RW;
+                // left neighbour of the next site (of site 0 the row's last one, old); site 0, new
+                uint32_t left = (row[RW - 1] >> ((L - 1) & 31)) & 1u, first = 0u;
+                for (int w = 0; w < RW; ++w) {
+                    const int n = min(32, L - 32 * w);
+                    uint32_t R = row[w];
+                    const uint32_t U = up[w], D = down[w], next = w + 1 < RW ? row[w + 1] & 1u : 0u;
+                    for (int j = 0; j < n; ++j, ++i) {
+                        if ((i & 3) == 0)
+                            blk = philox4x32_10(make_uint4((uint32_t)i >> 2, sweep, a.iteration, a.ctr3), a.key0,
+                                                (uint32_t)c);
+                        const uint32_t u = (i & 3) == 0 ? blk.x : (i & 3) == 1 ? blk.y : (i & 3) == 2 ? blk.z : blk.w;
+                        const uint32_t me = (R >> j) & 1u;
+                        const uint32_t right = j + 1 < n ? (R >> (j + 1)) & 1u : w + 1 < RW ? next : w == 0 ? R & 1u : first;
+                        const int unequal = (int)((right ^ me) + (left ^ me) + (((U >> j) & 1u) ^ me) + (((D >> j) & 1u) ^ me));
+                        const int b = (M + V) >> 1;
+                        const uint32_t A = a.thr[b * 10 + (me ? 5 : 0) + unequal];
+                        if (A == kAlways || u < A) {
+                            R ^= 1u << j;
+                            E += 8 - 4 * unequal;
+                            M -= me ? 2 : -2;
+                        }
+                        left = (R >> j) & 1u;
+                        if (HIST) {
+                            const int bn = (M + V) >> 1;
+                            if (SMEM_HIST)
+                                atomicAdd(&s_hist[bn], 1u);
+                            else
+                                atomicAdd(reinterpret_cast<unsigned long long *>(&a.H[bn]), 1ull);
+                        }
+                    }
+                    row[w] = R;
+                    if (w == 0) first = R & 1u;
                 }
             }
             if (a.E_rec) a.E_rec[(size_t)sw * a.rec_stride + c] = E;
