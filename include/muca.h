@@ -63,7 +63,10 @@ extern "C" {
 
 /* lattice staging of the sweep kernels */
 #define MUCA_STAGING_AUTO 0
-#define MUCA_STAGING_SHARED 1 /* lattices copied into shared memory for a launch */
+#define MUCA_STAGING_SHARED 1 /* lattices copied into shared memory for a launch; MUCA_ERR_ARG
+                                 where the lattices of 32 chains and the table and histogram
+                                 staged with them exceed 227 KB (Ising L > 162 but 204..226,
+                                 8-Potts L > 76) */
 #define MUCA_STAGING_GLOBAL 2 /* lattices stay in global memory (L2 / HBM) */
 
 /* ensembles: weights in the energy (multicanonical, Secs. 2-3) or, for the Ising

@@ -247,6 +247,7 @@ constexpr int kMaxSmem = 227 * 1024;
 // groups per block: 0 for as many as suit p (a batch's blocks have a fixed number)
 SweepPlan plan_sweeps(const muca_ctx *ctx, bool allow_compact = true, int groups = 0);
 SweepShape sweep_shape(const muca_ctx *ctx, const SweepPlan &pl, bool hist, int groups = 0);
+bool staging_fits(const SweepPlan &pl, const SweepShape &s);
 int hist_mode(const SweepPlan &pl);
 int plan_flags(const SweepPlan &pl);  // MUCA_PLAN_* bit mask
 constexpr int kBatchGroups = 4;       // groups of chains per work unit of a batch

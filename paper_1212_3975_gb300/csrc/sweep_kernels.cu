@@ -180,6 +180,14 @@ SweepShape sweep_shape(const muca_ctx *ctx, const SweepPlan &pl, bool hist, int 
     return s;
 }
 
+// Whether a launch may take its staging: the lattices of 32 chains beside the table and the
+// histogram, as callers know it (muca.h), and what the block that runs really takes (fewer
+// chains and a ring per group: it always fits where the first does).
+bool staging_fits(const SweepPlan &pl, const SweepShape &s)
+{
+    return pl.smem_bytes <= (size_t)kMaxSmem && s.smem <= (size_t)kMaxSmem;
+}
+
 SweepPlan plan_sweeps(const muca_ctx *ctx, bool allow_compact, int groups)
 {
     SweepPlan pl;
@@ -272,9 +280,9 @@ int launch_sweeps(muca_ctx *ctx, uint32_t phase, int n_sweeps, uint32_t sweep0, 
         int rc = launch_ktab(ctx);
         if (rc) return rc;
     }
-    if (pl.smem_bytes + 4 * sweep::ring_bytes(ctx->model) > (size_t)kMaxSmem)
-        return fail(MUCA_ERR_ARG, "shared-memory staging does not fit: " + std::to_string(pl.smem_bytes) + " bytes");
     const SweepShape shape = sweep_shape(ctx, pl, hist);
+    if (!staging_fits(pl, shape))
+        return fail(MUCA_ERR_ARG, "shared-memory staging does not fit: " + std::to_string(pl.smem_bytes) + " bytes");
     SweepArgs a;
     a.lat = ctx->d_lat;
     a.E = ctx->d_E;

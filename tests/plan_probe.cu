@@ -39,5 +39,16 @@ void probe_batch(int model, int L, int p, int out[2])
     out[1] = muca::batch_max_sweeps(&c);
 }
 
+// whether a standalone launch takes its staging; its shared memory and chains per block
+int probe_launch(int model, int L, int p, int staging, int chains_per_block, int hist, int out[2])
+{
+    const muca_ctx c = context(model, L, p, staging, chains_per_block);
+    const muca::SweepPlan pl = muca::plan_sweeps(&c);
+    const muca::SweepShape s = muca::sweep_shape(&c, pl, hist != 0);
+    out[0] = (int)s.smem;
+    out[1] = s.chains;
+    return muca::staging_fits(pl, s);
+}
+
 int probe_launches(int n_sweeps, int split, int most) { return muca::sweep_launches(n_sweeps, split, most); }
 }

@@ -1,11 +1,14 @@
 """Sizes of sweep launches, checked on the host over every lattice: 32-bit counts of a
-block stay below 2^31 whatever a batch is asked to do."""
+block stay below 2^31 whatever a batch is asked to do, and lattices are staged in shared
+memory wherever they fit."""
 import ctypes
 import os
 import subprocess
 
 import numpy as np
 import pytest
+
+import test_gpu_sweep_shapes as shapes
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ISING, POTTS = 0, 1
@@ -49,6 +52,20 @@ def test_batch_launches_keep_counts_in_32_bits(probe):
                 assert max(n * (s + 1) // k - n * s // k for s in (0, k // 2, k - 1)) <= most, (model, L, n, split)
 
 
+def test_staging_is_taken_where_it_fits(probe):
+    """Lattices in shared memory: every side whose 32 chains fit beside table and histogram
+    (a block holds fewer), and no other; automatic and global staging always."""
+    two = (ctypes.c_int * 2)()
+    takes = {ISING: set(range(4, 163, 2)) | set(range(204, 227, 2)), POTTS: set(range(3, 77))}
+    for model, L in SIDES:
+        for p in (1, 40, 4865, 20000):
+            for hist in (0, 1):
+                for staging in (0, 1, 2):
+                    ok = probe.probe_launch(model, L, p, staging, 0, hist, two)
+                    assert bool(ok) == (staging != 1 or L in takes[model]), (model, L, p, staging)
+                    assert not ok or (0 < two[0] <= 227 * 1024 and two[1] >= 1), (model, L, p, staging)
+
+
 @pytest.mark.gpu
 def test_batch_counts_all_attempts_of_a_cold_lattice(muca):
     """128 chains of a 4 x 4 lattice that stay in the ground state: more than 2^32 counts of
@@ -63,6 +80,13 @@ def test_batch_counts_all_attempts_of_a_cold_lattice(muca):
     b.close()
     assert int(H.sum()) == n * p * 16
     assert int(H.max()) > 2 ** 32
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("model,L", [(ISING, 4), (ISING, 20), (ISING, 66), (ISING, 162), (ISING, 226), (POTTS, 7),
+                                     (POTTS, 33), (POTTS, 70), (POTTS, 75), (POTTS, 76)])
+def test_lattices_in_shared_memory_bit_exact(muca, model, L):
+    shapes.test_every_shape_bit_exact(muca, model, L, 1)
 
 
 @pytest.mark.gpu
