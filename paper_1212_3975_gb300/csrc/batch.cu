@@ -275,7 +275,8 @@ int configure(muca_batch *b)
         const SweepPlan pl = plan_sweeps(c, false, kBatchGroups);
         const SweepShape shape = sweep_shape(c, pl, true, kBatchGroups);
         // (pairs wherever the table is in shared memory: run_unit)
-        if (shape.groups != kBatchGroups || (shape.lpc > 1 && pl.hist_pairs != pl.table_smem))
+        if (!staging_fits(pl, shape) || shape.groups != kBatchGroups ||
+            (shape.lpc > 1 && pl.hist_pairs != pl.table_smem))
             return fail(MUCA_ERR_ARG, "batched staging exceeds shared memory");
         BatchJob &j = b->h_jobs[i];
         j.model = c->model;

@@ -32,3 +32,26 @@ def test_a_smaller_batch_leaves_a_larger_one_its_shared_memory(muca):
     assert int(small.job(0).get_histogram().sum()) == 2 * 8 * 8 * 8
     small.close()
     large.close()
+
+
+@pytest.mark.parametrize("model,L,fits", [(ISING, 64, True), (ISING, 160, True), (ISING, 164, False),
+                                          (ISING, 224, True), (ISING, 256, False), (POTTS, 68, True),
+                                          (POTTS, 80, False), (POTTS, 128, False)])
+def test_batches_stage_what_single_contexts_stage(muca, model, L, fits):
+    """Lattices in shared memory: a batch and a context of its own take and refuse the same."""
+    q = 2 if model == ISING else 8
+    with muca.Muca(model, L, q, 3, 1, staging=1) as g:
+        if fits:
+            want = g.iterate(1)
+        else:
+            with pytest.raises(muca.MucaError):
+                g.iterate(1)
+    if not fits:
+        with pytest.raises(muca.MucaError) as ei:
+            muca.MucaBatch([(model, L, q, 3, 1)], staging=1)
+        assert ei.value.code == muca._muca.MUCA_ERR_ARG and "shared memory" in str(ei.value)
+        return
+    b = muca.MucaBatch([(model, L, q, 3, 1)], staging=1)
+    b.iterate(1, 1)
+    assert (b.job(0).get_histogram() == want).all()
+    b.close()
