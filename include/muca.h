@@ -78,7 +78,9 @@ extern "C" {
 typedef struct muca_config {
     int recursion;        /* MUCA_RECURSION_*; default accumulated */
     int correction_width; /* bins for the boundary slope (Sec. 3); 0 -> L */
-    int chains_per_block; /* multiple of 32, <= 256, or 0; the sweeps choose their own block shape */
+    int chains_per_block; /* chains per block of a sweep launch: a multiple of 32, <= 256 (or as many
+                             as twelve deciding warps and the shared memory hold); 0 -> automatic.
+                             Batches have work units of their own size. */
     int staging;          /* MUCA_STAGING_*; 0 -> automatic */
     int ensemble;         /* MUCA_ENSEMBLE_*; 0 -> energy */
     double beta;          /* inverse temperature of the multimagnetic ensemble */

@@ -139,7 +139,8 @@ int hist_mode(const SweepPlan &pl)
                                                                                            : sweep::kHistSingle;
 }
 
-// Groups per block (`groups` > 0: that many).  A pass takes some 680 cycles with one
+// Groups per block (`groups` > 0: that many; muca_config.chains_per_block > 0: its chains).
+// A pass takes some 680 cycles with one
 // deciding warp per scheduler, and 600 and 42 more per group with two or three (64 x 64:
 // 670 cycles in blocks of 4 groups, 845 of 6, 930 of 8, 1110 of 12); blocks beyond one per
 // SM wait for another wave.  (At 170 cycles per group more waves of smaller blocks were
@@ -159,6 +160,8 @@ SweepShape sweep_shape(const muca_ctx *ctx, const SweepPlan &pl, bool hist, int 
             return launch_smem(ctx, pl, false, true, G, s.lpc) <= (size_t)kMaxSmem;
         return pl.lattice_smem;
     };
+    if (groups <= 0 && ctx->cfg.chains_per_block > 0)  // the caller's, as far as there are so many warps and chains
+        groups = (int)std::min<long>(std::min<long>(ctx->cfg.chains_per_block * s.lpc / 32, sweep::kMaxGroups), all);
     int G = groups;
     if (groups <= 0) {
         double best = 0.0;

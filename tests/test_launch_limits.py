@@ -66,6 +66,23 @@ def test_staging_is_taken_where_it_fits(probe):
                     assert not ok or (0 < two[0] <= 227 * 1024 and two[1] >= 1), (model, L, p, staging)
 
 
+@pytest.mark.parametrize("model,L,per_warp", [(ISING, 8, 32), (ISING, 16, 32), (ISING, 18, 4), (ISING, 30, 4),
+                                              (ISING, 64, 2), (ISING, 66, 1), (ISING, 256, 1), (POTTS, 6, 16),
+                                              (POTTS, 16, 8), (POTTS, 32, 4), (POTTS, 33, 2), (POTTS, 128, 1)])
+def test_chains_per_block_is_the_callers(probe, model, L, per_warp):
+    """chains_per_block sets the block: that many chains, or what twelve deciding warps, the
+    chains there are and the shared memory allow."""
+    two = (ctypes.c_int * 2)()
+    for p in (5, 100, 3000, 20000):
+        for hist in (0, 1):
+            for cpb in (32, 64, 128, 256):
+                assert probe.probe_launch(model, L, p, 0, cpb, hist, two)
+                groups = min(cpb // per_warp, 12, -(-p // per_warp))
+                assert two[1] <= groups * per_warp and two[1] % per_warp == 0
+                # (a group takes at most 42 KB: fewer groups only where no other would fit)
+                assert two[1] == groups * per_warp or two[0] > (227 - 42) * 1024, (p, hist, cpb)
+
+
 @pytest.mark.gpu
 def test_batch_counts_all_attempts_of_a_cold_lattice(muca):
     """128 chains of a 4 x 4 lattice that stay in the ground state: more than 2^32 counts of
