@@ -48,7 +48,7 @@ extern "C" {
 #define MUCA_ERR_ARG (-1)     /* invalid argument or size */
 #define MUCA_ERR_CUDA (-2)    /* a CUDA call failed (message names it) */
 #define MUCA_ERR_OOM (-3)     /* device allocation failed */
-#define MUCA_ERR_TIMEOUT (-4) /* a bounded device wait gave up */
+#define MUCA_ERR_TIMEOUT (-4) /* a bounded loop of a kernel gave up: the chains are not valid until muca_reset */
 #define MUCA_ERR_STATE (-5)   /* call not valid in the context's current state */
 #define MUCA_ERR_IO (-6)      /* checkpoint file could not be read or written */
 

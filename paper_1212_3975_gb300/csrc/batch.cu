@@ -39,6 +39,7 @@ __device__ __forceinline__ SweepArgs batch_args(const BatchJob &j, int n_sweeps,
     a.H = j.H;
     a.E_rec = nullptr;
     a.M_rec = nullptr;
+    a.fault = j.fault;
     a.samples = nullptr;
     a.L = j.L;
     a.q = j.q;
@@ -308,6 +309,7 @@ int configure(muca_batch *b)
         j.iteration = b->d_iter + i;
         j.active = b->d_active + i;
         j.conv = b->d_conv + i;
+        j.fault = c->h_fault;
         j.ctr3_therm = ((uint32_t)(c->seed >> 32) << 2) | kPhaseThermalize;
         j.therm = b->d_therm + i;
         j.table_smem = pl.table_smem;
@@ -554,10 +556,9 @@ int begin_iterations(muca_batch *b)
     std::vector<uint32_t> it(b->n_jobs), th(b->n_jobs);
     for (int i = 0; i < b->n_jobs; ++i) {
         muca_ctx *c = b->ctx[i];
-        if (c->ktab_dirty) {
-            int rc = launch_ktab(c);
-            if (rc) return rc;
-        }
+        int rc = check_fault(c);
+        if (rc) return rc;
+        if (c->ktab_dirty && (rc = launch_ktab(c))) return rc;
         it[i] = c->iteration;
         th[i] = c->sweeps_therm;
     }
@@ -687,6 +688,8 @@ int muca_batch_converge(muca_batch *b, int n_sweeps, int therm_sweeps, int max_i
     MUCA_CUDA_TRY(cudaGetLastError());
     note_launches(1);
     MUCA_CUDA_TRY(cudaStreamSynchronize(b->stream));
+    for (muca_ctx *c : b->ctx)
+        if ((rc = check_fault(c))) return rc;
     return MUCA_OK;
 }
 

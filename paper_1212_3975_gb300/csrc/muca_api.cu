@@ -30,6 +30,12 @@ int cuda_fail(cudaError_t e, const char *what)
     return e == cudaErrorMemoryAllocation ? MUCA_ERR_OOM : MUCA_ERR_CUDA;
 }
 
+int check_fault(const muca_ctx *ctx)
+{
+    if (!*static_cast<const volatile int *>(ctx->h_fault)) return MUCA_OK;
+    return fail(MUCA_ERR_TIMEOUT, "a pass of a sweep did not settle: reset the context");
+}
+
 void note_launches(uint64_t n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
 bool alloc_should_fail()
@@ -91,6 +97,7 @@ int copy_out(muca_ctx *ctx, void *dst, const void *src, size_t bytes)
     } else {
         MUCA_CUDA_TRY(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, ctx->stream));
         MUCA_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+        return check_fault(ctx);
     }
     return MUCA_OK;
 }
@@ -164,10 +171,12 @@ int alloc_buffers(muca_ctx *c)
         return fail(MUCA_ERR_CUDA, "reweight scratch initialisation");
     }
     if (alloc_should_fail() ||
-        cudaMallocHost(reinterpret_cast<void **>(&c->h_stats), sizeof(muca_iter_stats)) != cudaSuccess) {
+        cudaMallocHost(reinterpret_cast<void **>(&c->h_stats), sizeof(muca_iter_stats) + sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
         return fail(MUCA_ERR_OOM, "pinned allocation failed");
     }
+    c->h_fault = reinterpret_cast<int *>(c->h_stats + 1);
+    *c->h_fault = 0;
     return MUCA_OK;
 }
 
@@ -316,6 +325,8 @@ int muca_reset(muca_ctx *ctx, uint64_t seed)
     ctx->samples_active = 0;
     ctx->lnw_version += 1;
     if ((rc = launch_init_lattice(ctx))) return rc;
+    // (the start clears the status; the next call asks for it on the host)
+    if (check_fault(ctx)) MUCA_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
     return launch_thresholds(ctx);
 }
 
@@ -362,6 +373,7 @@ int muca_update_weights(muca_ctx *ctx, muca_iter_stats *out)
         MUCA_CUDA_TRY(cudaMemcpyAsync(ctx->h_stats, ctx->d_stats, sizeof(muca_iter_stats), cudaMemcpyDeviceToHost,
                                       ctx->stream));
         MUCA_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+        if ((rc = check_fault(ctx))) return rc;
         if (out) *out = *ctx->h_stats;
     }
     if (log) {
@@ -594,6 +606,7 @@ int muca_get_energies(muca_ctx *ctx, int64_t *E, int64_t *M)
     MUCA_CUDA_TRY(cudaMemcpyAsync(e.data(), ctx->d_E, sizeof(int32_t) * ctx->p, cudaMemcpyDeviceToHost, ctx->stream));
     MUCA_CUDA_TRY(cudaMemcpyAsync(m.data(), ctx->d_M, sizeof(int32_t) * ctx->p, cudaMemcpyDeviceToHost, ctx->stream));
     MUCA_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+    if ((rc = check_fault(ctx))) return rc;
     for (int c = 0; c < ctx->p; ++c) {
         if (E) E[c] = e[c];
         if (M) M[c] = m[c];
@@ -719,6 +732,7 @@ int muca_save(muca_ctx *ctx, const char *path)
     h.lnw_version = ctx->lnw_version;
     h.samples_lnw_version = ctx->samples_lnw_version;
     MUCA_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+    if ((rc = check_fault(ctx))) return rc;
     FILE *f = std::fopen(path, "wb");
     if (!f) return fail(MUCA_ERR_IO, std::string("cannot open ") + path);
     bool ok = std::fwrite(&h, sizeof(h), 1, f) == 1;

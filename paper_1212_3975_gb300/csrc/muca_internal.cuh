@@ -94,6 +94,7 @@ struct SweepArgs {
     uint32_t ctr3;        // counter word 3 = (seed_hi << 2) | phase
     uint32_t key0;        // low 32 bits of the seed
     int rec_stride;       // records row stride (= p)
+    int *fault;           // set where a pass did not settle (muca_ctx::h_fault)
 };
 
 // staging of the sweep launches of a context
@@ -152,6 +153,7 @@ struct BatchJob {
     int table_smem, hist, lattice;  // staging of the sweep body (sweep_body.cuh)
     int lpc, row;               // lanes per chain; a row is one pass
     int *active;                // 0: the lattice is frozen (converged) and every batch kernel skips it
+    int *fault;                 // muca_ctx::h_fault
     int *conv;                  // iteration at which the lattice converged, -1 before
     uint32_t ctr3_therm;        // counter word 3 of thermalisation sweeps
     uint32_t *therm;            // device counter of thermalisation sweeps (counter word 1)
@@ -183,6 +185,7 @@ struct muca_ctx {
     uint64_t *d_samples;      // [3][n_bins]
     muca_iter_stats *d_stats;
     muca_iter_stats *h_stats; // pinned
+    int *h_fault;             // pinned, behind h_stats: set by a sweep whose pass did not settle
     // production series scratch (used when the caller passes host or null buffers)
     int32_t *d_series;        // [2][series_cap]
     size_t series_cap;        // records per array
@@ -209,6 +212,9 @@ namespace muca {
 int fail(int code, const std::string &msg);
 int cuda_fail(cudaError_t e, const char *what);
 void note_launches(uint64_t n);
+// MUCA_ERR_TIMEOUT if a sweep of the context gave up on a pass (the chains are then not
+// those of the method until a reset); asked before sweeps and after every wait for them
+int check_fault(const muca_ctx *ctx);
 
 // NVTX range around an entry point (visible in profilers; free without one attached)
 struct NvtxRange {

@@ -18,7 +18,9 @@
 //            resolved again.  Each repetition extends the agreeing prefix by at least one
 //            site (the first disagreeing site had the right history, so its test was
 //            exact), so this ends; thresholds of neighbouring bins differ by little, and
-//            most passes need no repair.
+//            most passes need no repair.  (A launch that repeats more than 4 LPC + 2 times
+//            per pass, which passes of 4 LPC sites cannot need, gives up and says so in
+//            a.fault.)
 //
 // Every decision is the exact integer test, so trajectories, histograms and records are
 // those of the site-by-site form, bit for bit.  Any predicted decisions give a real
@@ -489,6 +491,11 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
         const int flush_rows = HMODE == kHist16 ? max(1, 65535 / (lw * L)) : 0;
         const uint32_t rselw = ROW ? rsel_of(cl) : 0u, lselw = ROW ? lsel_of(cl) : 0u;
 
+        // repetitions that a launch may need at most (max_launch_sweeps keeps this an int).
+        // Beyond, no site is decided any more: a pass then agrees with itself and the launch
+        // ends.  (One allowance per launch and no exit of its own from the loop: a count per
+        // pass with a break took 3661 instead of 2967 us at 64 x 64, p = 14592.)
+        int left = passes * (4 * LPC + 2);
         for (int it = 0; it < passes; ++it) {
             const bool lastq = ROW || q == nq - 1;
             // ---- the next pass: what does not depend on this one's decisions
@@ -703,6 +710,10 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a, const int cblk, c
                         flip = flip1;
                     }
                     if (!__any_sync(~0u, bad != 0u)) break;
+                }
+                if (--left < 0) {
+                    if (lane == 0) *reinterpret_cast<volatile int *>(a.fault) = 1;
+                    vm = 0u;
                 }
                 // repair: the verified thresholds, for the left neighbours as met
 #pragma unroll

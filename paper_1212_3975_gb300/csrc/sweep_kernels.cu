@@ -15,8 +15,9 @@ namespace {
 // top bit is set.  Potts: the same words, s = (word * q) >> 32.
 // ---------------------------------------------------------------------------
 __global__ void init_lattice_kernel(uint32_t *lat, int model, int L, int q, int p, int p_pad, int row_words,
-                                    int lat_words, uint32_t key0, uint32_t ctr3)
+                                    int lat_words, uint32_t key0, uint32_t ctr3, int *fault)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *fault = 0;
     const size_t total = (size_t)lat_words * p_pad;
     for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
         const int c = (int)(t / lat_words), k = (int)(t % lat_words);
@@ -278,11 +279,10 @@ int launch_sweeps(muca_ctx *ctx, uint32_t phase, int n_sweeps, uint32_t sweep0, 
 {
     if (ctx->cfg.ensemble == MUCA_ENSEMBLE_MAGNETIZATION)
         return launch_muma_sweeps(ctx, phase, n_sweeps, sweep0, iteration, hist, E_rec, M_rec);
+    int rc = check_fault(ctx);
+    if (rc) return rc;
     const SweepPlan pl = plan_sweeps(ctx);
-    if (ctx->ktab_dirty) {
-        int rc = launch_ktab(ctx);
-        if (rc) return rc;
-    }
+    if (ctx->ktab_dirty && (rc = launch_ktab(ctx))) return rc;
     const SweepShape shape = sweep_shape(ctx, pl, hist);
     if (!staging_fits(pl, shape))
         return fail(MUCA_ERR_ARG, "shared-memory staging does not fit: " + std::to_string(pl.smem_bytes) + " bytes");
@@ -307,6 +307,7 @@ int launch_sweeps(muca_ctx *ctx, uint32_t phase, int n_sweeps, uint32_t sweep0, 
     a.ctr3 = ((uint32_t)(ctx->seed >> 32) << 2) | phase;
     a.key0 = (uint32_t)ctx->seed;
     a.rec_stride = ctx->p;
+    a.fault = ctx->h_fault;
     const int blocks = (ctx->p + shape.chains - 1) / shape.chains;
     // keep every block-histogram entry and draw position below 2^31
     const uint64_t per_sweep = (uint64_t)std::max(shape.chains, 32) * (ctx->V + 3);
@@ -330,7 +331,7 @@ int launch_init_lattice(muca_ctx *ctx)
     const int grid = (int)std::min<size_t>((size_t)ctx->n_sm * 16, (total + 127) / 128);
     init_lattice_kernel<<<grid, 128, 0, ctx->stream>>>(ctx->d_lat, ctx->model, ctx->L, ctx->q, ctx->p, ctx->p_pad,
                                                       ctx->row_words, ctx->lat_words, (uint32_t)ctx->seed,
-                                                      ((uint32_t)(ctx->seed >> 32) << 2) | kPhaseInit);
+                                                      ((uint32_t)(ctx->seed >> 32) << 2) | kPhaseInit, ctx->h_fault);
     MUCA_CUDA_TRY(cudaGetLastError());
     note_launches(1);
     return launch_recount(ctx);

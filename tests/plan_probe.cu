@@ -50,5 +50,13 @@ int probe_launch(int model, int L, int p, int staging, int chains_per_block, int
     return muca::staging_fits(pl, s);
 }
 
+// status of a context whose sweeps set `fault`
+int probe_fault(int fault)
+{
+    muca_ctx c = context(MUCA_ISING, 8, 1, MUCA_STAGING_AUTO, 0);
+    c.h_fault = &fault;
+    return muca::check_fault(&c);
+}
+
 int probe_launches(int n_sweeps, int split, int most) { return muca::sweep_launches(n_sweeps, split, most); }
 }

@@ -66,6 +66,13 @@ def test_staging_is_taken_where_it_fits(probe):
                     assert not ok or (0 < two[0] <= 227 * 1024 and two[1] >= 1), (model, L, p, staging)
 
 
+def test_a_pass_that_gives_up_is_an_error(probe):
+    """The status that a sweep leaves when a pass does not settle (which needs a mistake in
+    the kernel: no input brings it about)."""
+    assert probe.probe_fault(0) == 0
+    assert probe.probe_fault(1) == -4
+
+
 @pytest.mark.parametrize("model,L,per_warp", [(ISING, 8, 32), (ISING, 16, 32), (ISING, 18, 4), (ISING, 30, 4),
                                               (ISING, 64, 2), (ISING, 66, 1), (ISING, 256, 1), (POTTS, 6, 16),
                                               (POTTS, 16, 8), (POTTS, 32, 4), (POTTS, 33, 2), (POTTS, 128, 1)])
