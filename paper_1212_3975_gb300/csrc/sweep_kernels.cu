@@ -118,17 +118,51 @@ __global__ void unpack_kernel(const uint32_t *lat, int8_t *out, int model, int L
 }  // namespace
 
 namespace {
-// lanes per chain (1: the small-lattice body), and whether a row is one pass: the fewest
+// Cycles of a row with n groups per block, measured.  Rows decided at once: one deciding
+// warp per scheduler 680, two or three 600 and 42 per group (64 x 64: 670 in blocks of 4
+// groups, 845 of 6, 930 of 8, 1110 of 12).  A lane per chain (16 < L <= 32), per site: 61 to
+// 77 (18 x 18 to 32 x 32) with at most two deciding and two drawing warps on schedulers of
+// their own, 77 to 85 with three or four groups, 127 with 6, 144 with 8, 200 with 12.
+double row_cycles(int n) { return n <= 4 ? 680.0 : 600.0 + 42.0 * n; }
+double lane_row_cycles(int L, int n)
+{
+    return L * (n <= 2 ? 40.0 + 1.15 * L : n <= 4 ? 66.0 + 0.6 * L : 50.0 + 12.0 * n);
+}
+long waves_of(long groups, int per_block, int n_sm) { return ((groups + per_block - 1) / per_block + n_sm - 1) / n_sm; }
+
+// Whether a launch takes the body with a lane per chain.  Up to kSmallL always.  Up to
+// kLaneL a row's 18 to 32 sites one after the other take two to four times as long as the
+// row at once, but 32 chains per warp instead of four: with many chains the lattices of a
+// launch need fewer waves.  Both are costed, rows with a tenth more for repeated passes
+// (iterations of 2^16 sites with late weights, rows / lanes: 20 x 20, p = 7000 1918 / 2025
+// us, 9728 2870 / 1931, 16384 5192 / 2409; 32 x 32, p = 9728 2097 / 2432, 16384 3787 / 2661,
+// 29184 5455 / 4006).
+bool lane_per_chain(const muca_ctx *ctx, int groups)
+{
+    if (ctx->model != MUCA_ISING || ctx->L > sweep::kLaneL) return false;
+    if (ctx->L <= sweep::kSmallL) return true;
+    if (groups > 0 || ctx->cfg.staging == MUCA_STAGING_GLOBAL) return false;  // (batches; lattices not staged)
+    const long lanes = ((long)ctx->p + 31) / 32, rows = ((long)ctx->p + 3) / 4;
+    double lane_best = 1e30, row_best = 1e30;
+    for (int n = 1; n <= sweep::kMaxGroups; ++n) {
+        row_best = std::min(row_best, waves_of(rows, n, ctx->n_sm) * row_cycles(n));
+        if (sweep::small_smem(ctx->L, ctx->n_bins, ctx->lat_words, n, true) <= (size_t)kMaxSmem)
+            lane_best = std::min(lane_best, waves_of(lanes, n, ctx->n_sm) * lane_row_cycles(ctx->L, n));
+    }
+    return lane_best < 1.1 * row_best;
+}
+// lanes per chain (1: one, site by site), and whether a row is one pass: the fewest
 // lanes that hold a row of four sites per lane, so that no lane is idle in full launches
 // (8-Potts 8 x 8, p = 16384, 200 sweeps and an update: two lanes 1.20 ms, four 1.80)
-void lanes_of(int model, int L, int &lpc, bool &row)
+void lanes_of(const muca_ctx *ctx, int groups, int &lpc, bool &row)
 {
-    lpc = model == MUCA_ISING && L <= sweep::kSmallL ? 1 : L <= 8 ? 2 : L <= 16 ? 4 : L <= 32 ? 8 : L <= 64 ? 16 : 32;
+    const int L = ctx->L;
+    lpc = lane_per_chain(ctx, groups) ? 1 : L <= 8 ? 2 : L <= 16 ? 4 : L <= 32 ? 8 : L <= 64 ? 16 : 32;
     row = L <= 128;
 }
 size_t launch_smem(const muca_ctx *ctx, const SweepPlan &pl, bool hist, bool lattice, int groups, int lpc)
 {
-    if (lpc == 1) return sweep::small_smem(ctx->n_bins, ctx->lat_words, groups, hist);
+    if (lpc == 1) return sweep::small_smem(ctx->L, ctx->n_bins, ctx->lat_words, groups, hist);
     const size_t lat = lattice ? ((size_t)ctx->lat_words * 4 * (32 / lpc) * groups + 15) & ~(size_t)15 : 0;
     return pl.table_bytes + (hist ? pl.hist_bytes : 0) + lat + sweep::ring_bytes(ctx->model) * groups;
 }
@@ -140,20 +174,17 @@ int hist_mode(const SweepPlan &pl)
                                                                                            : sweep::kHistSingle;
 }
 
-// Groups per block (`groups` > 0: that many; muca_config.chains_per_block > 0: its chains).
-// A pass takes some 680 cycles with one
-// deciding warp per scheduler, and 600 and 42 more per group with two or three (64 x 64:
-// 670 cycles in blocks of 4 groups, 845 of 6, 930 of 8, 1110 of 12); blocks beyond one per
-// SM wait for another wave.  (At 170 cycles per group more waves of smaller blocks were
-// taken: 256 x 256, p = 8192, 6 waves of 9 groups 7.62 ms, 5 of 11 6.83 ms; 64 x 64,
-// p = 16000, 10 sweeps, 6 of 9 2.14 ms, 5 of 11 1.95 ms.)  Of equal costs the fewest
-// groups, on more SMs, deciding and drawing warps on schedulers of their own (8-Potts
-// 32 x 32, p = 639, 2 or 1 groups instead of 4: 413 against 530 us; 8 x 8, p = 1024:
-// 291 against 352).
+// Groups per block (`groups` > 0: that many; muca_config.chains_per_block > 0: its chains):
+// the fewest cycles over all waves, blocks beyond one per SM waiting for another wave.  (At
+// 170 cycles per group more waves of smaller blocks were taken: 256 x 256, p = 8192, 6 waves
+// of 9 groups 7.62 ms, 5 of 11 6.83 ms; 64 x 64, p = 16000, 10 sweeps, 6 of 9 2.14 ms, 5 of
+// 11 1.95 ms.)  Of equal costs the fewest groups, on more SMs, deciding and drawing warps on
+// schedulers of their own (8-Potts 32 x 32, p = 639, 2 or 1 groups instead of 4: 413 against
+// 530 us; 8 x 8, p = 1024: 291 against 352).
 SweepShape sweep_shape(const muca_ctx *ctx, const SweepPlan &pl, bool hist, int groups)
 {
     SweepShape s;
-    lanes_of(ctx->model, ctx->L, s.lpc, s.row);
+    lanes_of(ctx, groups, s.lpc, s.row);
     const long all = ((long)ctx->p * s.lpc + 31) / 32;
     auto staged = [&](int G) {
         // launches without a histogram stage the lattices in the room it leaves
@@ -168,8 +199,8 @@ SweepShape sweep_shape(const muca_ctx *ctx, const SweepPlan &pl, bool hist, int 
         double best = 0.0;
         for (int n = 1; n <= std::min<long>(sweep::kMaxGroups, all); ++n) {
             if (n > 1 && launch_smem(ctx, pl, hist, staged(n), n, s.lpc) > (size_t)kMaxSmem) break;
-            const long waves = ((all + n - 1) / n + ctx->n_sm - 1) / ctx->n_sm;
-            const double t = (double)waves * (n <= 4 ? 680.0 : 600.0 + 42.0 * n);
+            const double t = waves_of(all, n, ctx->n_sm) *
+                             (s.lpc == 1 && ctx->L > sweep::kSmallL ? lane_row_cycles(ctx->L, n) : row_cycles(n));
             if (best == 0.0 || t < best) {
                 best = t;
                 G = n;
@@ -198,9 +229,9 @@ SweepPlan plan_sweeps(const muca_ctx *ctx, bool allow_compact, int groups)
     const bool ising = ctx->model == MUCA_ISING;
     const int staging = ctx->cfg.staging, width = ktab_width(ctx->model);
     pl.compact = pl.t16 = pl.hist16 = pl.hist_pairs = false;
-    if (ising && ctx->L <= sweep::kSmallL) {  // the small-lattice body stages everything
+    if (lane_per_chain(ctx, groups)) {  // that body stages everything
         pl.table_smem = pl.hist_smem = pl.lattice_smem = true;
-        pl.smem_bytes = sweep::small_smem(ctx->n_bins, ctx->lat_words, 1, true);
+        pl.smem_bytes = sweep::small_smem(ctx->L, ctx->n_bins, ctx->lat_words, 1, true);
         pl.table_bytes = pl.hist_bytes = 0;  // (sizes of its own: launch_smem)
         return pl;
     }

@@ -71,6 +71,14 @@ cudaError_t launch_small(const SweepLaunch &l)
     case 12: return launch_small_as<12, HIST>(l);
     case 14: return launch_small_as<14, HIST>(l);
     case 16: return launch_small_as<16, HIST>(l);
+    case 18: return launch_small_as<18, HIST>(l);
+    case 20: return launch_small_as<20, HIST>(l);
+    case 22: return launch_small_as<22, HIST>(l);
+    case 24: return launch_small_as<24, HIST>(l);
+    case 26: return launch_small_as<26, HIST>(l);
+    case 28: return launch_small_as<28, HIST>(l);
+    case 30: return launch_small_as<30, HIST>(l);
+    case 32: return launch_small_as<32, HIST>(l);
     default: return cudaErrorInvalidConfiguration;
     }
 }

@@ -1,4 +1,5 @@
-// Ising sweep body of small lattices (L <= 16): one lane per chain, site by site.
+// Ising sweep body with one lane per chain, site by site: small lattices (L <= 16), and with
+// many chains every lattice of one word per row (L <= 32).
 //
 // A pass of sweep_body.cuh takes a chain of some 600 cycles however few its sites, so on
 // rows of up to 16 sites deciding one site after the other is faster (three iterations of
@@ -10,29 +11,45 @@
 // its start (draws, the neighbours of its first sites) is made during the row before: 61
 // cycles per site of 8 x 8 instead of 76, of which some 28 are instructions to issue.
 //
+// Longer rows (16 < L <= 32) take 61 to 77 cycles per site; 32 chains per warp make up for it
+// where a launch fills the GPU several times (lane_per_chain has the rule): 32 x 32,
+// p = 16384, 64 sweeps 2.66 ms against 3.79 of rows at once, 20 x 20 2.41 against 5.19.
+//
 // A block has G groups of 32 chains: warps 0..G-1 decide, up to four more draw the random
 // numbers into a ring per group (16 sites per hand-off).  Every lane has a histogram of its
 // own, count of bin b at word 32 b + lane: the chains of a warp share a few bins, and
-// atomics on one address wait on each other, and the table loads on them.
+// atomics on one address wait on each other, and the table loads on them.  (L > 16: one
+// histogram per block, with a count per lane or per two lanes.)
 #pragma once
 #include "sweep_body.cuh"
 
 namespace muca {
 namespace sweep {
 
-constexpr int kSmallL = 16;
+constexpr int kSmallL = 16;   // always in this body up to here
+constexpr int kLaneL = 32;    // with many chains up to here (one word per row)
 
-// Draws of a chain: three hand-offs of 16 sites, then the first again so that no row
-// wraps; 4 mod 32 words from chain to chain (vector loads of a warp hit every bank).
+// Draws of a chain, hand-offs of 16 sites.  Rows of up to 16 sites: three hand-offs, then
+// the first again so that no row wraps.  Longer rows: four (the row being loaded spans up to
+// three while the next is drawn), addressed modulo 64.  4 mod 32 words from chain to chain
+// (vector loads of a warp hit every bank).
 struct SmallRing {
-    static constexpr int kPhase = 16, kSites = 3 * kPhase, kStride = kSites + kPhase + 4;
+    static constexpr int kPhase = 16, kSites = 3 * kPhase, kWrap = 4 * kPhase, kStride = kWrap + 4;
     static constexpr size_t kBytes = 32 * kStride * 4;
 };
 
-// shared memory of a launch: table, histograms (one per lane), lattices, rings
-__host__ __device__ constexpr size_t small_smem(int n_bins, int lat_words, int groups, bool hist)
+// Counts per bin of a block's histogram, L > kSmallL: one per lane, or per two lanes where
+// one per lane would leave no room for twelve groups.  (24 x 24, p = 9728, 113 sweeps: eight
+// counts per bin 2868 us, 16 or 32 2048.)
+__host__ __device__ constexpr int lane_counts(int L) { return L <= 22 ? 32 : 16; }
+
+// shared memory of a launch: table, histograms (one per lane and group up to kSmallL; beyond,
+// lane_counts counts per bin for the block, and a word per lane for padding chains),
+// lattices, rings
+__host__ __device__ constexpr size_t small_smem(int L, int n_bins, int lat_words, int groups, bool hist)
 {
-    return (size_t)n_bins * 32 + ((hist ? (size_t)n_bins * 128 : 0) + (size_t)lat_words * 128 + SmallRing::kBytes) * groups;
+    const size_t h = !hist ? 0 : L <= kSmallL ? (size_t)n_bins * 128 * groups : (size_t)n_bins * 4 * lane_counts(L) + 128;
+    return (size_t)n_bins * 32 + h + ((size_t)lat_words * 128 + SmallRing::kBytes) * groups;
 }
 
 // Table offsets 4 n and row changes 64 - 32 n of four sites, one per byte, for the
@@ -60,14 +77,16 @@ template <int L, bool HIST>
 __device__ __forceinline__ void small_body(const SweepArgs &a, const int cblk, const int G, uint32_t *smem)
 {
     using Rg = SmallRing;
-    static_assert(L >= 4 && L <= kSmallL && L % 2 == 0, "small lattices");
+    static_assert(L >= 4 && L <= kLaneL && L % 2 == 0, "small lattices");
     constexpr int V = L * L, lat_words = L;
+    constexpr bool LONG = L > kSmallL;
     __syncthreads();  // (persistent kernel: smem may still be read by the previous unit)
     const int tid = threadIdx.x, nt = block_threads(G), lane = tid & 31, warp = tid >> 5;
     const int n_bins = a.n_bins, lw = 32 * G, c0 = cblk * lw;
     uint32_t *const s_tab = smem;
-    uint32_t *const s_hist = s_tab + 8 * n_bins;          // [G][n_bins][32]
-    const int n_hist = HIST ? 32 * n_bins * G : 0;
+    constexpr int C = lane_counts(L);                     // (LONG)
+    uint32_t *const s_hist = s_tab + 8 * n_bins;          // [G][n_bins][32], LONG: [n_bins][C], [32]
+    const int n_hist = !HIST ? 0 : LONG ? C * n_bins + 32 : 32 * n_bins * G;
     uint32_t *const s_lat = s_hist + n_hist;              // [lat_words][lw]
     uint32_t *const s_ring = s_lat + lat_words * lw;
     for (int i = tid; i < 8 * n_bins; i += nt) s_tab[i] = (i & 7) < 5 ? a.ktab[5 * (i >> 3) + (i & 7)] : 0u;
@@ -104,7 +123,7 @@ __device__ __forceinline__ void small_body(const SweepArgs &a, const int cblk, c
                     b.z = active ? min(b.z, 0xFFFFFFFEu) : 0xFFFFFFFFu;
                     b.w = active ? min(b.w, 0xFFFFFFFEu) : 0xFFFFFFFFu;
                     *reinterpret_cast<uint4 *>(ring + 4 * pass) = b;
-                    if (slot == 0) *reinterpret_cast<uint4 *>(ring + 4 * pass + Rg::kSites) = b;
+                    if (!LONG && slot == 0) *reinterpret_cast<uint4 *>(ring + 4 * pass + Rg::kSites) = b;
                     if (++qd == quads) {
                         qd = 0u;
                         ++ctr1;
@@ -114,7 +133,7 @@ __device__ __forceinline__ void small_body(const SweepArgs &a, const int cblk, c
             }
             qd0 = qd;
             ctr0 = ctr1;
-            slot = slot == 2 ? 0 : slot + 1;
+            slot = slot == (LONG ? 3 : 2) ? 0 : slot + 1;
         }
     } else {
         // ---------------- the chains ------------------------------------------------------------
@@ -125,8 +144,11 @@ __device__ __forceinline__ void small_body(const SweepArgs &a, const int cblk, c
         const uint32_t tab0 = (uint32_t)__cvta_generic_to_shared(s_tab);
         const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring_of(grp));
         const bool record = !HIST && (a.E_rec || a.M_rec || a.samples);
-        // (count of the row at P: word 32 (P - tab0) / 32 + lane)
-        const uint32_t hist0 = (uint32_t)__cvta_generic_to_shared(s_hist + 32 * n_bins * grp + lane) - 4u * tab0;
+        // (count of the row at P: word 32 (P - tab0) / 32 + lane, LONG: C (P - tab0) / 32 + lane % C;
+        // padding chains stay in one bin, and count it in the words behind)
+        constexpr uint32_t HS = LONG ? (uint32_t)C / 8u : 4u;
+        uint32_t hist0 = (uint32_t)__cvta_generic_to_shared(s_hist + (LONG ? lane % C : 32 * n_bins * grp + lane)) - HS * tab0;
+        if (LONG && !active) hist0 = (uint32_t)__cvta_generic_to_shared(s_hist + C * n_bins + lane) - HS * (tab0 + 32u * (V >> 1));
 
         // P0 / P1: table row before the site if the previous attempt was rejected / accepted
         // (ap: which); Q0 / Q1: the row after it if the site accepts, A0 / A1: the thresholds
@@ -148,7 +170,7 @@ __device__ __forceinline__ void small_body(const SweepArgs &a, const int cblk, c
         uint32_t u[L];
         constexpr int W = L % 4 == 0 ? 4 : 2;
         auto load_draws = [&](int j) {
-            const uint32_t us = ring_s + 4u * (uint32_t)(pos + j);
+            const uint32_t us = ring_s + 4u * (uint32_t)(LONG ? (pos + j) & (Rg::kWrap - 1) : pos + j);
             if constexpr (W == 4)
                 asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
                              : "=r"(u[j]), "=r"(u[j + 1]), "=r"(u[j + 2]), "=r"(u[j + 3])
@@ -157,10 +179,14 @@ __device__ __forceinline__ void small_body(const SweepArgs &a, const int cblk, c
                 asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(u[j]), "=r"(u[j + 1]) : "r"(us));
         };
         auto next_draws = [&] {
-            pos = pos + L >= Rg::kSites ? pos + L - Rg::kSites : pos + L;
+            pos = LONG ? (pos + L) & (Rg::kWrap - 1) : pos + L >= Rg::kSites ? pos + L - Rg::kSites : pos + L;
             lin += L;
         };
         bar_sync(1 + grp, 64);
+        if (LONG) {  // (two hand-offs: at least 324 sites are drawn)
+            bar_sync(1 + grp, 64);
+            next_sync += Rg::kPhase;
+        }
 #pragma unroll
         for (int j = 0; j < L; j += W) load_draws(j);
         next_draws();
@@ -171,10 +197,12 @@ __device__ __forceinline__ void small_body(const SweepArgs &a, const int cblk, c
         }
         for (int it = 0; it < rows; ++it) {
             // the next row's draws are handed off (past the last row: old ones, not used)
-            if (lin > next_sync) {
-                if (next_sync < phases * Rg::kPhase) bar_sync(1 + grp, 64);
-                next_sync += Rg::kPhase;
-            }
+#pragma unroll
+            for (int k = 0; k < (LONG ? 2 : 1); ++k)
+                if (lin > next_sync) {
+                    if (next_sync < phases * Rg::kPhase) bar_sync(1 + grp, 64);
+                    next_sync += Rg::kPhase;
+                }
             const int y1 = y + 1 == L ? 0 : y + 1;
             const uint32_t R1 = row_of(y1), D1w = row_of(y1 + 1 == L ? 0 : y1 + 1);
             const uint32_t ua = R ^ U, ub = R ^ D, tr = R ^ (R >> 1), q = R ^ (R << 1);
@@ -214,7 +242,7 @@ __device__ __forceinline__ void small_body(const SweepArgs &a, const int cblk, c
                     Q1 = (uint32_t)__dp4a((int)qd.D1, k, (int)Pa);
                 }
                 const bool acc = u[j] < (ap ? A1 : A0);
-                if (HIST) red_shared(hist0 + 4u * (acc ? Pa : Pc), 1u);
+                if (HIST) red_shared(hist0 + HS * (acc ? Pa : Pc), 1u);
                 Rw ^= acc ? 1u << j : 0u;
                 if (j == 0)  // the row's last site sees the updated site 0 to its right
                     last = ((ua >> (L - 1)) & 1u) + ((ub >> (L - 1)) & 1u) + (((R >> (L - 1)) ^ Rw) & 1u);
@@ -265,7 +293,14 @@ __device__ __forceinline__ void small_body(const SweepArgs &a, const int cblk, c
         const int k = i % lat_words, c = i / lat_words;
         if (c0 + c < a.p) a.lat[(size_t)c0 * lat_words + i] = s_lat[k * lw + c];
     }
-    if (HIST) {
+    if (HIST && LONG) {
+        for (int b = tid; b < n_bins; b += nt) {
+            uint32_t x = 0u;
+#pragma unroll
+            for (int i = 0; i < C; ++i) x += s_hist[C * b + (i + b) % C];
+            if (x) atomicAdd(reinterpret_cast<unsigned long long *>(a.H + b), (unsigned long long)x);
+        }
+    } else if (HIST) {
         // a warp per bin: counts of the block's chains (padding chains left out); all of a
         // launch's are below 2^31 (max_launch_sweeps)
         for (int b = warp; b < n_bins; b += nt >> 5) {

@@ -9,6 +9,7 @@ import numpy as np
 import pytest
 
 import test_gpu_sweep_shapes as shapes
+from oracle import MucaOracle, reweight
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ISING, POTTS = 0, 1
@@ -81,6 +82,8 @@ def test_chains_per_block_is_the_callers(probe, model, L, per_warp):
     chains there are and the shared memory allow."""
     two = (ctypes.c_int * 2)()
     for p in (5, 100, 3000, 20000):
+        if model == ISING and 16 < L <= 32 and p == 20000:
+            per_warp = 32  # (a lane per chain)
         for hist in (0, 1):
             for cpb in (32, 64, 128, 256):
                 assert probe.probe_launch(model, L, p, 0, cpb, hist, two)
@@ -88,6 +91,48 @@ def test_chains_per_block_is_the_callers(probe, model, L, per_warp):
                 assert two[1] <= groups * per_warp and two[1] % per_warp == 0
                 # (a group takes at most 42 KB: fewer groups only where no other would fit)
                 assert two[1] == groups * per_warp or two[0] > (227 - 42) * 1024, (p, hist, cpb)
+
+
+def test_many_chains_of_small_lattices_take_a_lane_each(probe):
+    """Ising sides of 18 to 32: rows at once (four chains per warp) with few chains, a lane
+    per chain with many; never in batches or with lattices in global memory."""
+    two = (ctypes.c_int * 2)()
+
+    def lanes(p, staging=0):
+        assert probe.probe_launch(ISING, L, p, staging, 0, 1, two)
+        assert two[0] <= 227 * 1024
+        return two[1] > 48  # (twelve warps of four chains)
+
+    for L in range(18, 33, 2):
+        assert not lanes(1000) and not lanes(4864), L
+        for p in (16384, 40000, 1 << 20):
+            assert lanes(p) and lanes(p, 1) and not lanes(p, 2), (L, p)
+        probe.probe_batch(ISING, L, 16384, two)
+        assert two[0] == 16, L
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("L", range(18, 33, 2))
+def test_a_lane_per_chain_bit_exact(muca, L):
+    """Iterations, thermalisation and records of more chains than fill the GPU's warps once,
+    a ragged last warp: every chain against the oracle."""
+    p = 16389
+    thr = shapes.noisy_thresholds(ISING, L)
+    with muca.Muca(ISING, L, 2, p, 21) as g:
+        g.set_thresholds(thr)
+        H1, H2 = g.iterate(2), g.iterate(1)
+        g.thermalize(1)
+        E, M = g.produce(2)
+        n, s1, s2 = g.get_samples()
+        spins = g.get_spins()
+    o = MucaOracle(ISING, L, 2, p, 21)
+    assert np.array_equal(H1, o.iterate(2, thr=thr)) and np.array_equal(H2, o.iterate(1, thr=thr))
+    o.thermalize(1, thr=thr)
+    e, m = o.produce(2, thr=thr)
+    assert np.array_equal(E, e) and np.array_equal(M, m)
+    for x, y in zip((n, s1, s2), reweight.bin_series(ISING, L, e, m)):
+        assert np.array_equal(x, y)
+    assert np.array_equal(spins, o.spins)
 
 
 @pytest.mark.gpu
