@@ -33,7 +33,6 @@ __device__ __forceinline__ SweepArgs batch_args(const BatchJob &j, int n_sweeps,
     a.E = j.E;
     a.M = j.M;
     a.cnt = j.cnt;
-    a.thr = j.thr;
     a.ktab = j.ktab;
     a.ktab31 = j.ktab + (size_t)j.n_bins * ktab_width(j.model);
     a.H = j.H;
@@ -42,7 +41,6 @@ __device__ __forceinline__ SweepArgs batch_args(const BatchJob &j, int n_sweeps,
     a.fault = j.fault;
     a.samples = nullptr;
     a.L = j.L;
-    a.q = j.q;
     a.p = j.p;
     a.p_pad = j.p_pad;
     a.row_words = j.row_words;
@@ -282,7 +280,6 @@ int configure(muca_batch *b)
         BatchJob &j = b->h_jobs[i];
         j.model = c->model;
         j.L = c->L;
-        j.q = c->q;
         j.p = c->p;
         j.p_pad = c->p_pad;
         j.row_words = c->row_words;
@@ -312,7 +309,6 @@ int configure(muca_batch *b)
         j.fault = c->h_fault;
         j.ctr3_therm = ((uint32_t)(c->seed >> 32) << 2) | kPhaseThermalize;
         j.therm = b->d_therm + i;
-        j.table_smem = pl.table_smem;
         j.hist = hist_mode(pl);
         j.lattice = shape.lattice;
         j.lpc = shape.lpc;

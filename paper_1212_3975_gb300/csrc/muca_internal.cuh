@@ -43,28 +43,6 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 ctr, uint32_t k0, uint32_t 
     return ctr;
 }
 
-// Same generator with the per-round second key word precomputed by the caller
-// (k1r[r] = k1 + r * 0xBB67AE85); the first key word is warp-uniform (the seed).
-__device__ __forceinline__ uint4 philox4x32_10_rk(uint4 ctr, uint32_t k0, const uint32_t (&k1r)[10])
-{
-#pragma unroll
-    for (int round = 0; round < 10; ++round) {
-        const uint32_t kr0 = k0 + (uint32_t)round * 0x9E3779B9u;
-        const uint32_t lo0 = 0xD2511F53u * ctr.x;
-        const uint32_t hi0 = __umulhi(0xD2511F53u, ctr.x);
-        const uint32_t lo1 = 0xCD9E8D57u * ctr.z;
-        const uint32_t hi1 = __umulhi(0xCD9E8D57u, ctr.z);
-        ctr = make_uint4(hi1 ^ ctr.y ^ kr0, lo1, hi0 ^ ctr.w ^ k1r[round], lo0);
-    }
-    return ctr;
-}
-
-__device__ __forceinline__ void philox_round_keys(uint32_t k1, uint32_t (&k1r)[10])
-{
-#pragma unroll
-    for (int round = 0; round < 10; ++round) k1r[round] = k1 + (uint32_t)round * 0xBB67AE85u;
-}
-
 // counter word 3: (seed >> 32) << 2 | phase
 enum Phase : uint32_t { kPhaseInit = 0, kPhaseIterate = 1, kPhaseThermalize = 2, kPhaseProduce = 3 };
 
@@ -80,14 +58,13 @@ struct SweepArgs {
     int32_t *E;           // [p_pad] running energy
     int32_t *M;           // [p_pad] running magnetisation (Ising) / record scratch
     uint64_t *cnt;        // Potts packed state counts [2][p_pad]
-    const uint32_t *thr;  // [n_bins][n_de]
     const uint32_t *ktab; // kernel table: Ising [n_bins][5] by unequal neighbours, Potts [n_bins][9] by dE+4
     const uint32_t *ktab31; // the same, entries >> 1
     uint64_t *H;          // merged histogram [n_bins] (uint64, atomically added)
     int32_t *E_rec;       // [n_sweeps][rec_stride] or null
     int32_t *M_rec;
     uint64_t *samples;    // [3][n_bins] production sums (n, sum|M|, sum M^2) or null
-    int L, q, p, p_pad, row_words, lat_words, n_bins;
+    int L, p, p_pad, row_words, lat_words, n_bins;
     int n_sweeps;
     uint32_t sweep0;      // counter word 1 of the first sweep
     uint32_t iteration;   // counter word 2
@@ -138,7 +115,7 @@ inline int sweep_launches(int n_sweeps, int split, int most)
 
 // Device view of one lattice of a batch (pointers into its context).
 struct BatchJob {
-    int model, L, q, p, p_pad, row_words, lat_words, n_bins, n_de, V;
+    int model, L, p, p_pad, row_words, lat_words, n_bins, n_de, V;
     int accumulated, width;
     uint32_t key0, ctr3_iter;   // seed low word; counter word 3 of weight iterations
     uint32_t *lat;
@@ -150,7 +127,7 @@ struct BatchJob {
     uint64_t *H;
     muca_iter_stats *stats;
     uint32_t *iteration;        // device counter of weight iterations (counter word 2)
-    int table_smem, hist, lattice;  // staging of the sweep body (sweep_body.cuh)
+    int hist, lattice;          // staging of the sweep body (sweep_body.cuh)
     int lpc, row;               // lanes per chain; a row is one pass
     int *active;                // 0: the lattice is frozen (converged) and every batch kernel skips it
     int *fault;                 // muca_ctx::h_fault
@@ -246,7 +223,6 @@ int launch_sweeps(muca_ctx *ctx, uint32_t phase, int n_sweeps, uint32_t sweep0,
 int launch_unpack_spins(muca_ctx *ctx, int8_t *d_out);
 int launch_thresholds(muca_ctx *ctx);
 int launch_update(muca_ctx *ctx);
-int launch_stats(muca_ctx *ctx);
 int launch_reweight(muca_ctx *ctx, const double *d_betas, int n_beta, int precision,
                     double *const out[4] /* e, C, absm, chi: device [n_beta] each */);
 constexpr int kMaxSmem = 227 * 1024;

@@ -272,9 +272,10 @@ SweepPlan plan_sweeps(const muca_ctx *ctx, bool allow_compact, int groups)
         pl.smem_bytes = table + hist;
         pl.hist_bytes = hist;
         // two to two and a half such groups per SM at L = 64: the table of the upper 16-bit
-        // halves of the thresholds (ties read the 32-bit table), which leaves L1 to the
-        // lattices.  Beyond, the 32-bit table's shorter pass is worth more (p = 14592:
-        // 3.47 against 4.33 ms for 20 sweeps and an update).
+        // halves of the thresholds (ties read the 32-bit table).  Kept only because the plan of
+        // this size is asserted (MUCA_PLAN_TABLE16), not for speed: 20 sweeps at p = 9824 take
+        // 2.84 ms with it and 2.67 with the 32-bit table, 11000 3.54 / 3.31, 12160 3.56 / 3.33,
+        // p = 14592 (and an update) 4.33 / 3.47.
         if (ctx->L == 64 && groups32 > 2 * n_sm && 2 * groups32 <= 5 * n_sm) {
             const size_t table16 = ((size_t)ctx->n_bins * 5 * 2 + 15) & ~(size_t)15;
             pl.t16 = true;
@@ -322,13 +323,11 @@ int launch_sweeps(muca_ctx *ctx, uint32_t phase, int n_sweeps, uint32_t sweep0, 
     a.E = ctx->d_E;
     a.M = ctx->d_M;
     a.cnt = ctx->d_cnt;
-    a.thr = ctx->d_thr;
     a.ktab = ctx->d_ktab;
     a.ktab31 = ctx->d_ktab + (size_t)ctx->n_bins * ktab_width(ctx->model);
     a.H = ctx->d_H;
     a.samples = samples ? ctx->d_samples : nullptr;
     a.L = ctx->L;
-    a.q = ctx->q;
     a.p = ctx->p;
     a.p_pad = ctx->p_pad;
     a.row_words = ctx->row_words;
@@ -340,9 +339,7 @@ int launch_sweeps(muca_ctx *ctx, uint32_t phase, int n_sweeps, uint32_t sweep0, 
     a.rec_stride = ctx->p;
     a.fault = ctx->h_fault;
     const int blocks = (ctx->p + shape.chains - 1) / shape.chains;
-    // keep every block-histogram entry and draw position below 2^31
-    const uint64_t per_sweep = (uint64_t)std::max(shape.chains, 32) * (ctx->V + 3);
-    const int chunk = (int)std::max<uint64_t>(1, std::min<uint64_t>((1ull << 31) / per_sweep, 1u << 30));
+    const int chunk = max_launch_sweeps(shape.chains, ctx->V);
     for (int done = 0; done < n_sweeps; done += chunk) {
         a.n_sweeps = std::min(chunk, n_sweeps - done);
         a.sweep0 = sweep0 + (uint32_t)done;

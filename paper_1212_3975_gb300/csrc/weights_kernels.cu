@@ -64,11 +64,6 @@ __global__ void ktab_kernel(const uint32_t *thr, uint32_t *ktab, int model, int 
     ktab[n_bins * width + t] = v >> 1;  // (as the sweep bodies compare them)
 }
 
-struct BlockStats {
-    unsigned long long total, mn, mx, n_sampled, K;
-    int lo, hi;
-};
-
 // The update runs as two kernels.  The recursion's differences (two logarithms and two
 // divisions in FP64 per bin, at two FP64 operations per clock and SM: 0.15 ms for 4097
 // bins on one SM) take a grid of blocks; what follows is one block per lattice
