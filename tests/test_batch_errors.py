@@ -55,3 +55,20 @@ def test_batches_stage_what_single_contexts_stage(muca, model, L, fits):
     b.iterate(1, 1)
     assert (b.job(0).get_histogram() == want).all()
     b.close()
+
+
+@pytest.mark.parametrize("job", [(ISING, 132, 2, 5, 2), (ISING, 224, 2, 3, 2), (ISING, 240, 2, 9, 2), (ISING, 256, 2, 6, 2),
+                                 (ISING, 260, 2, 5, 2), (ISING, 292, 2, 2, 2), (POTTS, 132, 8, 5, 2), (POTTS, 160, 8, 3, 2)])
+def test_long_rows_in_a_batch(muca, job):
+    """Rows of several passes and every histogram of theirs (32-bit and 16-bit counts in shared
+    memory, global): a batch and a context of its own agree bit for bit."""
+    b = muca.MucaBatch([job, (ISING, 8, 2, 8, 1)])
+    b.iterate(2, 2)
+    with muca.Muca(*job) as g:
+        for _ in range(2):
+            H = g.iterate(2)
+            g.update_weights()
+        v = b.job(0)
+        assert (v.get_histogram() == H).all() and (v.get_lnw() == g.get_lnw()).all()
+        assert (v.get_spins() == g.get_spins()).all()
+    b.close()
