@@ -54,17 +54,17 @@ SWEEP_SOURCES = ["paper_1212_3975_gb300/csrc/" + f for f in
 COUNTERS = {
     # Ising 64x64, p = 1024 (128 blocks of four groups of two chains):
     # profiles/ising_ws_sweep_L64_p1024.md
-    "ising_L64": {"source": "f205e94c2f0b658f", "inst_per_attempt": 2.669, "shared_wavefronts_per_attempt": 0.390,
+    "ising_L64": {"source": "959e22f09ee2b742", "inst_per_attempt": 2.669, "shared_wavefronts_per_attempt": 0.390,
                   "traffic_bytes_per_launch": 645376},
     # Ising 64x64, more groups of 32 chains than SMs (p = 9728):
     # profiles/ising_ws_compact_L64_p9728.md
-    "ising_L64_compact": {"source": "f205e94c2f0b658f", "inst_per_attempt": 2.538, "shared_wavefronts_per_attempt": 0.362,
-                          "traffic_bytes_per_launch": 6116608},
+    "ising_L64_compact": {"source": "959e22f09ee2b742", "inst_per_attempt": 2.538, "shared_wavefronts_per_attempt": 0.362,
+                          "traffic_bytes_per_launch": 6132736},
     # Ising 64x64, 16-bit table (p = 9824): profiles/ising_ws_t16_L64_p14592.md
-    "ising_L64_t16": {"source": "f205e94c2f0b658f", "inst_per_attempt": 2.696, "shared_wavefronts_per_attempt": 0.341,
-                      "traffic_bytes_per_launch": 6266624},
+    "ising_L64_t16": {"source": "959e22f09ee2b742", "inst_per_attempt": 2.696, "shared_wavefronts_per_attempt": 0.341,
+                      "traffic_bytes_per_launch": 6197504},
     # 8-Potts 32x32, p = 4096: profiles/potts_ws_sweep_L32_p4096.md
-    "potts_L32": {"source": "f205e94c2f0b658f", "inst_per_attempt": 3.517, "shared_wavefronts_per_attempt": 0.560,
+    "potts_L32": {"source": "959e22f09ee2b742", "inst_per_attempt": 3.517, "shared_wavefronts_per_attempt": 0.560,
                   "traffic_bytes_per_launch": 4324352},
 }
 # Cycles of one pass of a group alone on its SM (64 sites of an Ising row at L = 64, 32 of an

@@ -89,8 +89,13 @@ __device__ __forceinline__ void small_body(const SweepArgs &a, const int cblk, c
     const int n_hist = !HIST ? 0 : LONG ? C * n_bins + 32 : 32 * n_bins * G;
     uint32_t *const s_lat = s_hist + n_hist;              // [lat_words][lw]
     uint32_t *const s_ring = s_lat + lat_words * lw;
+    // (many loads in flight per thread: a block may have two warps only.  One 16 x 16 sweep of
+    // 8 chains took 45 us with a load at a time here and a warp per bin at the end, 24 now; of
+    // 8 x 8 18 and 12)
+#pragma unroll 16
     for (int i = tid; i < 8 * n_bins; i += nt) s_tab[i] = (i & 7) < 5 ? a.ktab[5 * (i >> 3) + (i & 7)] : 0u;
-    for (int i = tid; i < n_hist; i += nt) s_hist[i] = 0u;
+    for (int i = tid; i < n_hist / 4; i += nt) reinterpret_cast<uint4 *>(s_hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll 8
     for (int i = tid; i < lat_words * lw; i += nt) {
         const int k = i % lat_words, c = i / lat_words;
         s_lat[k * lw + c] = c0 + c < a.p ? a.lat[(size_t)c0 * lat_words + i] : 0u;
@@ -301,14 +306,20 @@ __device__ __forceinline__ void small_body(const SweepArgs &a, const int cblk, c
             if (x) atomicAdd(reinterpret_cast<unsigned long long *>(a.H + b), (unsigned long long)x);
         }
     } else if (HIST) {
-        // a warp per bin: counts of the block's chains (padding chains left out); all of a
+        // a thread per bin: counts of the block's chains (padding chains left out); all of a
         // launch's are below 2^31 (max_launch_sweeps)
-        for (int b = warp; b < n_bins; b += nt >> 5) {
+        for (int b = tid; b < n_bins; b += nt) {
             uint32_t x = 0u;
-            for (int g = 0; g < G; ++g)
-                if (c0 + 32 * g + lane < a.p) x += s_hist[32 * (n_bins * g + b) + lane];
-            x = __reduce_add_sync(~0u, x);
-            if (lane == 0 && x) atomicAdd(reinterpret_cast<unsigned long long *>(a.H + b), (unsigned long long)x);
+            for (int g = 0; g < G; ++g) {
+                const int n = a.p - c0 - 32 * g;  // chains of the group, or more
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    const int k = (i + b) & 31;
+                    const uint32_t v = s_hist[32 * (n_bins * g + b) + k];
+                    x += k < n ? v : 0u;
+                }
+            }
+            if (x) atomicAdd(reinterpret_cast<unsigned long long *>(a.H + b), (unsigned long long)x);
         }
     }
 }
