@@ -35,7 +35,7 @@
 // the sampled range the observables come from bins of relative weight ~1e-12, i.e.
 // |a| ~ 40 (log2 units), where a single float exponent would carry a relative error of
 // ~|a| 2^-24 into those weights.  Column sums are float pairs (an error-free addition
-// per term) within a thread and a warp, FP64 across warps and chunks.
+// per term) within a thread, a warp and a block, FP64 across chunks.
 //
 // MUCA_BF16 (muca_reweight only): one block of 8 warps per tile of 16 betas (the M
 // dimension of mma.m16n8k16), an FP64 prologue per tile (reference bin, window,
@@ -700,7 +700,7 @@ __device__ __forceinline__ int halving_index(int lane)
 // Tiles whose exponents reach too far take the exponential of every term.  FP32:
 // compensated exponents and weights in FP32; every column sum is kept as a float pair
 // (high part and the accumulated rounding errors of its additions), through the thread's
-// bins and the warp's sums, and combined in FP64 across warps.  (Plain FP32 sums of 32
+// bins, the warp's sums and the block's; chunks are added in FP64.  (Plain FP32 sums of 32
 // terms lost up to ~1e-6 relative on C and chi.)
 // Bound by the FP64 pipe (two per clock and SM; ~12 per term, besides exponentials and
 // sums) and by instruction issue in FP32 (~70 per term).  512 betas on the 4097 bins of

@@ -39,8 +39,8 @@ struct SmallRing {
 };
 
 // Counts per bin of a block's histogram, L > kSmallL: one per lane, or per two lanes where
-// one per lane would leave no room for twelve groups.  (24 x 24, p = 9728, 113 sweeps: eight
-// counts per bin 2868 us, 16 or 32 2048.)
+// one per lane would leave no room for twelve groups.  (28 x 28, p = 9728, 83 sweeps: eight
+// counts per bin 3059 us, 16 2237, 32 2203; p = 58368 16 6520, 32 7929.)
 __host__ __device__ constexpr int lane_counts(int L) { return L <= 22 ? 32 : 16; }
 
 // shared memory of a launch: table, histograms (one per lane and group up to kSmallL; beyond,
